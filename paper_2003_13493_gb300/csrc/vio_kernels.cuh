@@ -436,17 +436,39 @@ __device__ __forceinline__ uint32_t sad_b(const uint8_t* __restrict__ p) {
     return s;
 }
 
-// Byte-wise |a - b| > t for the 4 pixels of a word, without carries between
-// bytes: with k7 = 127 - t (t < 128), (d & 0x7F) + k7 carries into bit 7 iff
-// (d & 0x7F) > t, and a set bit 7 of d alone means d >= 128 > t; with
-// k7 = 255 - t (t >= 128) the carry means (d & 0x7F) > t - 128, which counts
-// only together with bit 7 of d.  The flags are bit 7 of each byte; the
-// other bits are left over and cleared by the caller.
+// Byte-wise |a - b| > t for the 4 pixels of a word: bit 7 of each byte, the
+// other bits clear.  Never misses a pixel, and for t < 128 may flag one with
+// |a - b| == t: with k7 = 127 - t the sum d + k7 reaches bit 7 when d > t, or
+// d >= 128 holds bit 7 itself; a byte that overflows (d > 128 + t) carries 1
+// into its neighbour, which changes that neighbour's flag only at d == t.
+// The coarse test keeps a superset anyway and the full test decides, so the
+// mask that would stop the carry is left out (one instruction in four).  With
+// t >= 128 a byte that overflowed would lose its flag: there (d & 0x7F) is
+// added to k7 = 255 - t, the carry into bit 7 means (d & 0x7F) > t - 128, and
+// it counts only together with bit 7 of d (exact).
 template <bool HIGH_T>
 __device__ __forceinline__ uint32_t gt_flags(uint32_t a, uint32_t b, uint32_t k7) {
     const uint32_t d = __vabsdiffu4(a, b);
-    const uint32_t f = (d & 0x7F7F7F7Fu) + k7;
-    return HIGH_T ? (f & d) : (f | d);
+    return HIGH_T ? (((d & 0x7F7F7F7Fu) + k7) & d & 0x80808080u) : (((d + k7) | d) & 0x80808080u);
+}
+
+// Appends a row's flags to a word of eight rows: the rows move down one bit
+// in their bytes, the oldest falls out, the new row enters at bit 7.
+__device__ __forceinline__ uint32_t push_row(uint32_t acc, uint32_t flags) {
+    return ((acc >> 1) & 0x7F7F7F7Fu) | flags;
+}
+
+// Pixels with RUN cyclically consecutive flags among the eight even circle
+// points f (N NE E SE S SW W NW), 32 pixels per word.
+template <int RUN>
+__device__ __forceinline__ uint32_t run_of_even(const uint32_t (&f)[8]) {
+    static_assert(RUN == 5 || RUN == 6, "two runs of three that overlap or meet");
+    uint32_t r3[8], keep = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) r3[i] = f[i] & f[(i + 1) & 7] & f[(i + 2) & 7];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) keep |= r3[i] & r3[(i + RUN - 3) & 7];
+    return keep;
 }
 
 // ---------------------------------------------------------------------------
@@ -462,8 +484,8 @@ __device__ __forceinline__ uint32_t gt_flags(uint32_t a, uint32_t b, uint32_t k7
 //      TH+2R+6) into one of two image buffers; the other buffer is loading
 //      the next item meanwhile.
 //   2. Coarse test on every score-region pixel of the warp's band, 4 pixels
-//      per lane (the 8-point rule for arcs n <= 11 and R <= 2, else the
-//      compass rule), pixels outside the testable area masked off; one warp
+//      per lane (runs of the eight even circle points), pixels outside the
+//      testable area masked off; one warp
 //      scan places each lane's kept pixels in the warp's queue, written by a
 //      two-ended bit walk as raw codes (coarse_and_compact).
 //   3. Each warp runs the full segment test on its queue and compacts the
@@ -545,119 +567,135 @@ __device__ __forceinline__ int walk_code_index(uint32_t code, int r0) {
 __device__ __forceinline__ uint32_t nibble(uint32_t keep) { return (keep * 0x00204081u) >> 28; }
 
 // Coarse test (the CCRF of Algorithm 1) over this warp's score rows,
-// appending the kept pixels (score-region index row * 128 + column) to the
-// warp's queue; returns the queue length.
+// appending the kept pixels (as raw walk codes) to the warp's queue; returns
+// the queue length.
 //
 // Warp w owns the 2*PPW score rows starting at r0 = 2*PPW*w; lane l owns the
 // 4-pixel word of score columns 4l .. 4l+3 in every one of them, so a row is
 // one conflict-free 128-byte read per warp.  The rule: an arc of n >= 9
-// contiguous points contains floor(n/4) >= 2 cyclically consecutive compass
-// points (0, 4, 8, 12), all darker or all brighter and so all with
-// |I_x - I_c| > t; a pixel is kept when two adjacent compass points (n <= 11)
-// or three of the four (n >= 12) differ from the centre by more than t.  With
-// EIGHT (n <= 11, NMS radius <= 2) the stronger rule on the eight even
-// circle points (compass points and the (+-2, +-2) diagonals) applies: an arc
-// of n >= 9 holds floor(n/2) >= 4 cyclically consecutive even points, so a
-// pixel is kept when four consecutive of the eight differ by more than t.
-// Neither rule drops a corner.
+// contiguous points holds floor(n/2) cyclically consecutive of the eight even
+// circle points (compass points and the (+-2, +-2) diagonals), all darker or
+// all brighter and so all with |I_x - I_c| > t.  A pixel is kept when 4 (n =
+// 9), 5 (n = 10, 11) or 6 (n >= 12) consecutive even points differ from the
+// centre by more than t; without EIGHT, when two adjacent compass points do.
+// No corner is dropped.  On the mixed batch's recipe at t = 10, n = 10 the run
+// of 5 keeps 4.9 % of the level-0 pixels where the two compass points keep
+// 19.5 %; at t = 20, n = 12 the run of 6 keeps 0.2 / 3.4 / 10 % of levels
+// 0 / 1 / 2 where three compass points keep 0.9 / 8.7 / 22 %.
 //
 // Each comparison is made once and serves two pixels: rows y and y+3 of a
 // column give the S flag of row y and the N flag of row y+3; columns x and
-// x+3 of a row give the E flag of x and the W flag of x+3 (the W flags of a
-// word come from the E flags of the word to its left, a lane shuffle away);
-// likewise (x, y)-(x+2, y+2) is SE of the first and NW of the second, and
-// (x, y)-(x-2, y+2) is SW of the first and NE of the second.  The shuffles
-// leave the outermost columns of lanes 0 and 31 without the left or right
-// neighbour word; those columns are outside the NMS region for radius 1
-// (lane 0's W flags of columns 0..2) and radius <= 2 (the diagonal flags of
-// columns 0, 1, 126, 127), so a radius of 2 reads the left word for its W
-// flags and radii >= 3 use the compass rule on every level.
+// x+3 of a row give the E flag of x and the W flag of x+3; (x, y)-(x+2, y+2)
+// is SE of the first and NW of the second, and (x, y)-(x+2, y-2) is NE of the
+// first and SW of the second.  A row thus costs two word loads, two byte
+// permutes and four compares.  The flags of a lane gather in words of eight
+// rows (bit 8j + i = row i, column 4l + j), so the second pixel's flags are
+// the same words a few rows later (one running word per comparison,
+// read at two points) and, where the columns differ, byte-permuted with the
+// word of the lane to the left: three shuffles and the rule itself once per
+// eight rows instead of once per row.  The kernel is bound by the ALU pipe
+// (logic, shifts, permutes: one instruction every two cycles) and by issue,
+// and this test is half of its ALU work: with the rule and the shuffles per
+// row the mixed batch took 107.1 M warp instructions and 133.7 us, so 94.0 M
+// and 117.5 us; 9x9 NMS at n = 10 on 16 frames 67.6 -> 52.8 us a call.
+// Lane 0 has no lane to its left: its W flags of columns 0..2 and NW / SW
+// flags of columns 0, 1 count as set, which keeps more, never fewer.
 //
-// The kept-pixel bits of a lane gather in 32-bit words, eight rows per
-// word (bit 8j + i of word w = row r0 + 8w + i, column 4l + j: each row's
-// flags, bit 7 of each byte, enter at the top and move down one bit per
-// row); one warp scan of the popcounts places each lane's run in the queue,
-// and each lane writes its pixels by walking its set bits, from both ends
+// One warp scan of the popcounts places each lane's run in the queue, and each
+// lane writes its pixels by walking its set bits, from both ends
 // at once, as raw codes.  (Spreading the
 // bits over the warp first, by a skewed bit transpose, balances the walk but
 // scatters the queue, and the full test's circle reads then conflict in
 // shared memory: slower.)
 // vm: bit 7 of byte j set when column 4l + j is inside the columns NMS reads.
-template <bool HIGH_T, bool THREE, int TH, int R, bool EIGHT = false>
+template <bool HIGH_T, int TH, int R, bool EIGHT = true>
 __device__ __forceinline__ int coarse_and_compact(const uint8_t* img, uint16_t* queue, int xw, uint32_t k7,
-                                                  int warp, int lane, int row_lo, int row_hi, uint32_t vm,
+                                                  int n_arc, int warp, int lane, int row_lo, int row_hi, uint32_t vm,
                                                   uint32_t* status = nullptr) {
     using G = TileGeom<TH, R>;
     constexpr int RW = G::BW / 4;      // words per box row
     constexpr int RPW = 2 * G::PPW;    // score rows per warp
-    constexpr int NW = (4 * RPW + 31) / 32;  // mask words per lane
-    static_assert(!EIGHT || R <= 2, "the diagonal flags of the edge lanes cover NMS radii <= 2");
+    constexpr int NW = (RPW + 7) / 8;  // mask words per lane
+    static_assert(RPW == 4 || RPW % 8 == 0, "a word holds eight rows, or the only four");
     constexpr uint32_t kFull = 0xFFFFFFFFu;
     const int r0 = RPW * warp;
+    // a band with no testable row (below or above the level) keeps nothing
+    if (row_hi <= r0 || row_lo >= r0 + RPW) return 0;
     // this lane's word in box row r0 (score row r is box row r + 3)
     const uint32_t* col = reinterpret_cast<const uint32_t*>(img) + r0 * RW + xw + lane;
-    uint32_t m[NW];
-#pragma unroll
-    for (int w = 0; w < NW; ++w) m[w] = 0u;
-    // One pass down the rows: step jj reads box row r0 + jj (C[jj]), forms
-    // the comparisons that row completes, and emits score row i = jj - 6,
-    // whose flags are then all known:
-    //   Dv[j]: box rows j and j + 3 (S flags of box row j, N flags of j + 3);
-    //   D1[j] / D2[j]: box row j against the pixels 2 right / 2 left of row
-    //   j + 2 (SE / SW flags of row j, NW / NE flags of row j + 2).
-    uint32_t C[RPW + 6], Dv[RPW + 3], D1[RPW + 3], D2[RPW + 3];
+    // One pass down the rows: step jj reads box row r0 + jj and makes the
+    // comparisons that it completes.  wv holds the vertical ones of box rows
+    // (i, i+3), w1 and w2 the diagonal ones of box rows (i+1, i+3), we the
+    // horizontal ones of box row i + 3, for i up to jj - 3.
+    uint32_t C[RPW + 6], R2[RPW + 6];
+    uint32_t wv = 0u, w1 = 0u, w2 = 0u, we = 0u;
+    uint32_t fn[NW], fs[NW], fe[NW], fne[NW], fse[NW], fsw[NW], fnw[NW];
 #pragma unroll
     for (int jj = 0; jj < RPW + 6; ++jj) {
         C[jj] = col[jj * RW];
-        if (jj >= 3) Dv[jj - 3] = gt_flags<HIGH_T>(C[jj - 3], C[jj], k7);
-        if (EIGHT && jj >= 3 && jj - 2 < RPW + 3) {
-            const int j = jj - 2;
-            const uint32_t r2 = col[jj * RW + 1];
-            const uint32_t l2 = __shfl_up_sync(kFull, C[jj], 1);
-            D1[j] = gt_flags<HIGH_T>(C[j], __byte_perm(C[jj], r2, 0x5432), k7);
-            D2[j] = gt_flags<HIGH_T>(C[j], __byte_perm(l2, C[jj], 0x5432), k7);
+        uint32_t rw = 0u;
+        if ((EIGHT && jj >= 1 && jj < RPW + 5) || (jj >= 3 && jj < RPW + 3)) rw = col[jj * RW + 1];
+        if (EIGHT) R2[jj] = __byte_perm(C[jj], rw, 0x5432);
+        if (jj < 3) continue;
+        const int i = jj - 3;
+        // the flags of score rows 8w .. 8w+7 are complete (and at the top of
+        // the word) once the row that holds row 8w + 7, or the last, is in
+        const auto done = [](int row) { return row >= 0 && row < RPW && ((row & 7) == 7 || row == RPW - 1); };
+        wv = push_row(wv, gt_flags<HIGH_T>(C[i], C[jj], k7));
+        if (done(i)) fn[i / 8] = wv;
+        if (done(i - 3)) fs[(i - 3) / 8] = wv;
+        if (i < RPW) {
+            we = push_row(we, gt_flags<HIGH_T>(C[jj], __byte_perm(C[jj], rw, 0x6543), k7));
+            if (done(i)) fe[i / 8] = we;
         }
-        if (jj < 6) continue;
-        const int i = jj - 6;  // score row r0 + i is box row r0 + j
-        const int j = i + 3;
-        const uint32_t c = C[j];
-        const uint32_t rw = col[j * RW + 1];
-        // E flags of this word; W flags from the E flags of the word to the left
-        const uint32_t fe = gt_flags<HIGH_T>(c, __byte_perm(c, rw, 0x6543), k7);
-        uint32_t el;
-        if (R == 1) {
-            el = __shfl_up_sync(kFull, fe, 1);
-        } else {
-            const uint32_t lw = col[j * RW - 1];
-            el = gt_flags<HIGH_T>(lw, __byte_perm(lw, c, 0x6543), k7);
+        if (EIGHT && i < RPW + 2) {
+            w1 = push_row(w1, gt_flags<HIGH_T>(C[jj - 2], R2[jj], k7));
+            w2 = push_row(w2, gt_flags<HIGH_T>(C[jj], R2[jj - 2], k7));
+            if (done(i)) {
+                fnw[i / 8] = w1;
+                fne[i / 8] = w2;
+            }
+            if (done(i - 2)) {
+                fse[(i - 2) / 8] = w1;
+                fsw[(i - 2) / 8] = w2;
+            }
         }
-        const uint32_t fw = __byte_perm(el, fe, 0x4321);
-        const uint32_t fn = Dv[i], fs = Dv[j];
-        uint32_t keep;
-        if (EIGHT) {
-            const uint32_t fse = D1[j], fsw = D2[j];
-            const uint32_t fnw = __byte_perm(__shfl_up_sync(kFull, D1[j - 2], 1), D1[j - 2], 0x5432);
-            const uint32_t fne = __byte_perm(D2[j - 2], __shfl_down_sync(kFull, D2[j - 2], 1), 0x5432);
-            // the 8 runs of four on the cycle N NE E SE S SW W NW, grouped by
-            // their middle three around a diagonal
-            const uint32_t xne = fn & fne & fe, xse = fe & fse & fs, xsw = fs & fsw & fw, xnw = fw & fnw & fn;
-            keep = ((xne | xsw) & (fse | fnw)) | ((xse | xnw) & (fne | fsw));
-        } else if (THREE) {  // at least 3 of 4 (any 3 of 4 cyclic positions are consecutive)
-            keep = (fn & fe & (fs | fw)) | (fs & fw & (fn | fe));
-        } else {             // two adjacent: (N|S) & (E|W)
-            keep = (fn | fs) & (fe | fw);
-        }
-        // row i of word i / 8 lands in bit i % 8 of each byte after the
-        // remaining shifts of that word: bit 8j + (i % 8) = row, column 4l + j
-        m[i / 8] = (m[i / 8] >> 1) | (keep & 0x80808080u);
     }
-    // a last word of fewer than 8 rows: its first row down to bit 0
-    if (RPW % 8) m[NW - 1] >>= 8 - RPW % 8;
+    uint32_t m[NW];
+#pragma unroll
+    for (int w = 0; w < NW; ++w) {
+        // columns x - 3 and x - 2 of the flags that belong to the pixel on their right
+        const auto from_left = [&](uint32_t f) {
+            const uint32_t l = __shfl_up_sync(kFull, f, 1);
+            return lane == 0 ? kFull : l;
+        };
+        const uint32_t fw = __byte_perm(from_left(fe[w]), fe[w], 0x4321);
+        if (EIGHT) {
+            const uint32_t nw = __byte_perm(from_left(fnw[w]), fnw[w], 0x5432);
+            const uint32_t sw = __byte_perm(from_left(fsw[w]), fsw[w], 0x5432);
+            const uint32_t f[8] = {fn[w], fne[w], fe[w], fse[w], fs[w], sw, fw, nw};
+            if (n_arc == 9) {  // uniform
+                // the 8 runs of four, grouped by their middle three around a diagonal
+                const uint32_t xne = f[0] & f[1] & f[2], xse = f[2] & f[3] & f[4], xsw = f[4] & f[5] & f[6],
+                               xnw = f[6] & f[7] & f[0];
+                m[w] = ((xne | xsw) & (f[3] | f[7])) | ((xse | xnw) & (f[1] | f[5]));
+            } else if (n_arc < 12) {
+                m[w] = run_of_even<5>(f);
+            } else {
+                m[w] = run_of_even<6>(f);
+            }
+        } else {  // two adjacent: (N|S) & (E|W)
+            m[w] = (fn[w] | fs[w]) & (fe[w] | fw);
+        }
+    }
+    // a word of four rows holds them in the upper half of each byte
+    if constexpr (RPW < 8) m[0] >>= 8 - RPW;
     // rows outside the testable area and columns outside the NMS region
     const uint32_t cols = ((vm >> 7) & 0x01010101u) * 0xFFu;
 #pragma unroll
     for (int w = 0; w < NW; ++w) {
-        const int lo = min(max(row_lo - r0 - 8 * w, 0), 8), hi = min(max(row_hi - r0 - 8 * w, 0), 8);
+        constexpr int kRows = RPW < 8 ? RPW : 8;
+        const int lo = min(max(row_lo - r0 - 8 * w, 0), 8), hi = min(max(row_hi - r0 - 8 * w, 0), kRows);
         const uint32_t rows = ((0xFFu << lo) & ~(0xFFu << hi) & 0xFFu) * 0x01010101u;
         m[w] &= rows & cols;
     }
@@ -880,7 +918,6 @@ __global__ void __launch_bounds__(kThreads, 4) fast_nms_cell_kernel(const uint8_
     const uint32_t lt_mask = (1u << lane) - 1u;
     const int thresh = cv.h->thresh, n_arc = cv.h->arc;
     const bool high_t = thresh >= 128;
-    const bool three = n_arc >= 12;
     const uint32_t k7 = (uint32_t)((high_t ? 255 : 127) - thresh) * 0x01010101u;
 
     for (int t = 0;; ++t) {
@@ -908,15 +945,8 @@ __global__ void __launch_bounds__(kThreads, 4) fast_nms_cell_kernel(const uint8_
             const uint32_t vm = (cols4 + (uint32_t)(0x80 - in.xlo) * 0x01010101u) &
                                 ~(cols4 + (uint32_t)(0x80 - in.xhi) * 0x01010101u) & 0x80808080u;
             const int xw = xoff / 4;
-            // the 8-point test (n <= 11 and NMS radius <= 2; n >= 12 keeps 3 of 4)
-            constexpr bool kEight = R <= 2;
-            if (!three) {
-                total = high_t ? coarse_and_compact<true, false, TH, R, kEight>(img, queue, xw, k7, warp, lane, row_lo, row_hi, vm, status)
-                               : coarse_and_compact<false, false, TH, R, kEight>(img, queue, xw, k7, warp, lane, row_lo, row_hi, vm, status);
-            } else {
-                total = high_t ? coarse_and_compact<true, true, TH, R>(img, queue, xw, k7, warp, lane, row_lo, row_hi, vm, status)
-                               : coarse_and_compact<false, true, TH, R>(img, queue, xw, k7, warp, lane, row_lo, row_hi, vm, status);
-            }
+            total = high_t ? coarse_and_compact<true, TH, R>(img, queue, xw, k7, n_arc, warp, lane, row_lo, row_hi, vm, status)
+                           : coarse_and_compact<false, TH, R>(img, queue, xw, k7, n_arc, warp, lane, row_lo, row_hi, vm, status);
         }
         __syncwarp();
 

@@ -173,16 +173,17 @@ __global__ void __launch_bounds__(kThreads, 3) fast_sweep_kernel(const uint8_t* 
             const uint32_t vm = (cols4 + (uint32_t)(0x80 - in.xlo) * 0x01010101u) &
                                 ~(cols4 + (uint32_t)(0x80 - in.xhi) * 0x01010101u) & 0x80808080u;
             const int xw = xoff / 4;
-            // levels >= 1: the 8-point test, also a necessary condition for every arc length
+            // levels >= 1: the run of even circle points that the shortest
+            // arc needs; level 0, where few pixels pass at all: two compass points
             if (k > 0)
-                total = high_t ? coarse_and_compact<true, false, TH, 1, true>(img, queue, xw, k7, warp, lane, row_lo,
+                total = high_t ? coarse_and_compact<true, TH, 1>(img, queue, xw, k7, arc_min, warp, lane, row_lo,
                                                                               row_hi, vm, status)
-                               : coarse_and_compact<false, false, TH, 1, true>(img, queue, xw, k7, warp, lane, row_lo,
+                               : coarse_and_compact<false, TH, 1>(img, queue, xw, k7, arc_min, warp, lane, row_lo,
                                                                                row_hi, vm, status);
             else
-                total = high_t ? coarse_and_compact<true, false, TH, 1>(img, queue, xw, k7, warp, lane, row_lo,
+                total = high_t ? coarse_and_compact<true, TH, 1, false>(img, queue, xw, k7, arc_min, warp, lane, row_lo,
                                                                          row_hi, vm, status)
-                               : coarse_and_compact<false, false, TH, 1>(img, queue, xw, k7, warp, lane, row_lo,
+                               : coarse_and_compact<false, TH, 1, false>(img, queue, xw, k7, arc_min, warp, lane, row_lo,
                                                                           row_hi, vm, status);
         }
         __syncwarp();
