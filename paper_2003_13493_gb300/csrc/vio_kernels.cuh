@@ -524,11 +524,6 @@ struct TileGeom {
 constexpr int kConsumers = 256;             // 8 warps that detect
 constexpr int kThreads = kConsumers + 32;   // + 1 producer warp (items, TMA)
 
-// A work item decoded from its index: item i of the call's tile table.
-struct Item {
-    int frame, level, tx, ty;
-};
-
 // What the consumers need of an item, written by the producer next to the
 // image buffer it fills.
 struct ItemInfo {
@@ -541,19 +536,18 @@ struct ItemInfo {
     uint64_t* keys;
 };
 
-// Item i of the call's tile table: entry j = (L-1-k)*n + f (coarsest level first).
-__device__ __forceinline__ Item decode_item(const CallView& cv, const int32_t* tiles, int it) {
-    const int n = cv.h->n_frames, L = cv.h->levels;
-    const int j = upper_index(tiles, n * L, it);
-    Item r;
-    r.frame = j % n;
-    r.level = L - 1 - j / n;
-    const int t = it - tiles[j];
-    const int wk = cv.fds[r.frame].w >> r.level;
-    const int ntx = (wk + kTileW - 1) / kTileW;
-    r.ty = t / ntx;
-    r.tx = t - r.ty * ntx;
-    return r;
+// upper_index by a whole warp (all lanes call it with the same arguments):
+// 32 entries per step, so 1024 entries take two dependent loads instead of ten.
+__device__ __forceinline__ int upper_index_warp(const int32_t* a, int n, int v, int lane) {
+    int lo = 0, len = n;
+    while (len > 1) {  // the answer lies in [lo, lo + len)
+        const int step = (len + 31) / 32, o = lane * step;
+        const uint32_t le = __ballot_sync(0xFFFFFFFFu, o < len && a[lo + o] <= v);
+        const int k = 31 - __clz(le);  // a[lo] <= v: bit 0 is set
+        lo += k * step;
+        len = min(step, len - k * step);
+    }
+    return lo;
 }
 
 // Score-region index of a raw walk code (w << 10 | lane << 5 | bit b) of the
@@ -771,59 +765,87 @@ __device__ __forceinline__ bool own_rows_reset(uint64_t* nms_bars, int t, T* til
     return true;
 }
 
-// Producer of the detect kernels (one thread): claims work items from the
-// counter one ahead of their use, decodes each into the tile it covers and
-// issues the TMA load of the tile and its halo into the next buffer of the
-// ring once the consumer warps have released it.  An item index >= n_items
-// tells the consumers to stop.
+// Producer of the detect kernels (one warp): takes work items (the CTA's own
+// index first, then from the counter, claimed one ahead of their use), decodes
+// each into the tile it covers, and issues the TMA load of the tile and its
+// halo into the next buffer of the ring once the consumer warps have released
+// it.  An item index >= n_items tells the consumers to stop.
+//
+// Decoding is a chain of dependent loads (the tile table, the frame), about
+// 2,400 cycles by one thread and after the release, which the consumers then
+// waited for on top of the load itself: 2,100 of 7,950 cycles per tile on 4K
+// frames with few corners.  It is done by the warp and before the wait for the
+// release (8 4K frames, FAST-12: 107.5 -> 101.8 us a call; 64 mixed frames
+// 148.3 -> 145.5 us).
+//
+// The pyramid's levels are written by the kernel before this one, which may
+// still be running (programmatic dependent launch); a level-0 tile reads the
+// caller's frame and need not wait for it, unless that kernel also uploads the
+// frame.
 template <int TH, int R>
 __device__ __forceinline__ void produce_tiles(const CallView& cv, const int32_t* tiles, int32_t* counter,
                                               uint32_t* status, ItemInfo* info, uint64_t* full_bar,
-                                              uint64_t* empty_bar, uint8_t* smem) {
+                                              uint64_t* empty_bar, uint8_t* smem, int lane) {
     using G = TileGeom<TH, R>;
     constexpr int NB = G::NBUF;
-    const int n_items = cv.h->n_items;
-    int claimed = atomicAdd(counter, 1);
+    const int n_items = cv.h->n_items, n = cv.h->n_frames, L = cv.h->levels;
+    int claimed = 0;  // lane 0's
+    bool pyramid_done = false;
     for (int t = 0;; ++t) {
         const int b = t % NB;
-        const int it = claimed;
-        if (it < n_items) claimed = atomicAdd(counter, 1);
-        if (t >= NB && !mbar_wait_bounded(&empty_bar[b], ((t / NB) - 1) & 1, kWaitLimitNs)) {
-            atomicOr(status, kStatusTimeout);
-            return;
-        }
-        ItemInfo& in = info[b];
+        const int it = t == 0 ? (int)blockIdx.x : (int)gridDim.x + __shfl_sync(0xFFFFFFFFu, claimed, 0);
+        if (lane == 0 && it < n_items) claimed = atomicAdd(counter, 1);
+        ItemInfo in = {};
         in.id = it;
-        if (it >= n_items) {
-            mbar_arrive(&full_bar[b]);
+        const CUtensorMap* map = nullptr;
+        if (it < n_items) {
+            // entry j = (L-1-k) * n + f of the tile table (coarsest level first)
+            const int j = upper_index_warp(tiles, n * L, it, lane);
+            const int f = j % n;
+            in.level = L - 1 - j / n;
+            const FrameDesc& fd = cv.fds[f];
+            const uint8_t* uploaded = fd.src0;
+            in.gw = fd.gw;
+            in.gh = fd.gh;
+            in.keys = fd.keys;
+            in.wk = fd.w >> in.level;
+            in.hk = fd.h >> in.level;
+            in.magic = cv.h->cell_magic[in.level];
+            const int ti = it - tiles[j], ntx = (in.wk + kTileW - 1) / kTileW;
+            const int ty = ti / ntx;
+            in.x0 = (ti - ty * ntx) * G::TW;
+            in.y0 = ty * TH;
+            // per-item constants, computed once here instead of by every
+            // consumer warp: score column 0 is level x = x0 - 4 and box column
+            // 0 is (x0 - 8) & ~15; score row r is level y = y0 - R + r; testable
+            // pixels are 3 <= x < Wk - 3, 3 <= y < Hk - 3; the NMS reads score
+            // columns 4 - R .. 123 + R only
+            in.xoff = in.x0 - 4 - ((in.x0 - 8) & ~15);
+            in.row_lo = max(0, 3 - in.y0 + R);
+            in.row_hi = min(G::SR, in.hk - 3 - in.y0 + R);
+            in.xlo = max(4 - R, 7 - in.x0);
+            in.xhi = min(124 + R, in.wk + 1 - in.x0);
+            map = in.level == 0 ? &cv.maps0[f] : &cv.mapsk[f * (kMaxLevels - 1) + in.level - 1];
+            if (lane == 0) fence_tensormap_acquire(map);
+            if (!pyramid_done && (in.level > 0 || uploaded)) {
+                griddep_wait();
+                pyramid_done = true;
+            }
+        }
+        if (t >= NB && !mbar_wait_bounded(&empty_bar[b], ((t / NB) - 1) & 1, kWaitLimitNs)) {
+            if (lane == 0) atomicOr(status, kStatusTimeout);
             return;
         }
-        const Item wi = decode_item(cv, tiles, it);
-        const FrameDesc& fd = cv.fds[wi.frame];
-        in.level = wi.level;
-        in.x0 = wi.tx * G::TW;
-        in.y0 = wi.ty * TH;
-        in.wk = fd.w >> wi.level;
-        in.hk = fd.h >> wi.level;
-        in.gw = fd.gw;
-        in.gh = fd.gh;
-        in.keys = fd.keys;
-        // per-item constants, computed once here instead of by every
-        // consumer warp: score column 0 is level x = x0 - 4 and box column
-        // 0 is (x0 - 8) & ~15; score row r is level y = y0 - R + r; testable
-        // pixels are 3 <= x < Wk - 3, 3 <= y < Hk - 3; the NMS reads score
-        // columns 4 - R .. 123 + R only
-        in.magic = cv.h->cell_magic[wi.level];
-        in.xoff = in.x0 - 4 - ((in.x0 - 8) & ~15);
-        in.row_lo = max(0, 3 - in.y0 + R);
-        in.row_hi = min(G::SR, in.hk - 3 - in.y0 + R);
-        in.xlo = max(4 - R, 7 - in.x0);
-        in.xhi = min(124 + R, in.wk + 1 - in.x0);
-        const CUtensorMap* map =
-            wi.level == 0 ? &cv.maps0[wi.frame] : &cv.mapsk[wi.frame * (kMaxLevels - 1) + wi.level - 1];
-        fence_tensormap_acquire(map);
-        mbar_arrive_expect_tx(&full_bar[b], G::BOX);
-        tma_load_2d(smem + G::IMG_OFF + b * G::BOXA, map, &full_bar[b], (in.x0 - 8) & ~15, in.y0 - R - 3);
+        if (lane == 0) {
+            info[b] = in;
+            if (it >= n_items) {
+                mbar_arrive(&full_bar[b]);
+            } else {
+                mbar_arrive_expect_tx(&full_bar[b], G::BOX);
+                tma_load_2d(smem + G::IMG_OFF + b * G::BOXA, map, &full_bar[b], (in.x0 - 8) & ~15, in.y0 - R - 3);
+            }
+        }
+        if (it >= n_items) return;
     }
 }
 
@@ -904,12 +926,7 @@ __global__ void __launch_bounds__(kThreads, 4) fast_nms_cell_kernel(const uint8_
 
     griddep_launch_dependents();
     if (warp == kConsumers / 32) {
-        // the pyramid levels the tiles read are written by the kernel before
-        // this one, which may still be running (programmatic dependent launch)
-        if (lane == 0) {
-            griddep_wait();
-            produce_tiles<TH, R>(cv, cached ? tiles_sh : cv.tiles, counter, status, info, full_bar, empty_bar, smem);
-        }
+        produce_tiles<TH, R>(cv, cached ? tiles_sh : cv.tiles, counter, status, info, full_bar, empty_bar, smem, lane);
         return;
     }
 

@@ -103,8 +103,7 @@ __global__ void __launch_bounds__(kThreads, 3) fast_sweep_kernel(const uint8_t* 
     __syncthreads();
 
     if (warp == kConsumers / 32) {
-        if (lane == 0) produce_tiles<TH, 1>(cv, cached ? tiles_sh : cv.tiles, counter, status, info, full_bar, empty_bar,
-                                            smem);
+        produce_tiles<TH, 1>(cv, cached ? tiles_sh : cv.tiles, counter, status, info, full_bar, empty_bar, smem, lane);
         return;
     }
 
