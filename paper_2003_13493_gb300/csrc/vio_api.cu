@@ -57,6 +57,7 @@ int first_variant(int r) {
 
 PyrFn pyr_fn(int levels) {
     switch (levels) {
+        case 1: return pyramid_kernel<1>;
         case 2: return pyramid_kernel<2>;
         case 3: return pyramid_kernel<3>;
         case 4: return pyramid_kernel<4>;
@@ -202,7 +203,7 @@ vio_status enqueue_kernels(vio_ctx* ctx, int variant, int levels, cudaStream_t s
     if (prof) VIO_CK(cudaStreamIsCapturing(s, &cap));
     const unsigned rec_flags = cap == cudaStreamCaptureStatusActive ? cudaEventRecordExternal : 0u;
     if (prof) VIO_CK(cudaEventRecordWithFlags(ctx->stage_ev[0], s, rec_flags));
-    if (levels > 1 && pyramid) {
+    if (pyramid) {
         pyr_fn(levels)<<<ctx->sm_count * (small ? 1 : 8), 256, 0, s>>>(ctx->d_call);
         VIO_CK(cudaGetLastError());
     }
@@ -235,8 +236,9 @@ vio_status enqueue_kernels(vio_ctx* ctx, int variant, int levels, cudaStream_t s
     return VIO_OK;
 }
 
-// Graph slot `levels` holds pyramid -> detect -> decode; slot 0 holds
-// detect -> decode alone (the pyramid is already in place).
+// Graph slot `levels` holds pyramid -> detect -> decode (with one level the
+// pyramid kernel only stages frames); slot 0 holds detect -> decode alone (the
+// pyramid is already in place, or there is nothing to build or stage).
 vio_status get_graph(vio_ctx* ctx, int variant, int levels, bool pyramid, bool small, int ctas,
                      cudaGraphExec_t* out) {
     cudaGraphExec_t& g = ctx->graphs[variant][pyramid ? levels : 0][small ? 1 : 0][ctas];
@@ -260,9 +262,9 @@ vio_status get_graph(vio_ctx* ctx, int variant, int levels, bool pyramid, bool s
 
 // Lays the batch out in the resident arenas, fills the call block, uploads
 // it and launches the three kernels on `s`.
-// Frames that the pyramid kernel uploads itself: src[i] non-null is the
-// device mapping of frame i in host memory (row pitch pitch[i]); lev0[i] is
-// then the device copy that kernel writes.
+// Frames that the pyramid kernel uploads or stages itself: src[i] non-null is
+// frame i (row pitch pitch[i]) as the device mapping of host memory or as device
+// memory that TMA cannot address; lev0[i] is then the copy that kernel writes.
 struct Upload {
     const uint8_t* const* src = nullptr;
     const int* pitch = nullptr;
@@ -364,7 +366,7 @@ constexpr int kZeroCopyMin = 4;  // lone pinned frames per call read through the
 vio_status enqueue_sweep(vio_ctx* ctx, int levels, cudaStream_t s, bool pyramid, const SweepInfo* d_sw) {
     const bool prof = ctx->cfg.profile != 0;
     if (prof) VIO_CK(cudaEventRecord(ctx->stage_ev[0], s));
-    if (levels > 1 && pyramid) {
+    if (pyramid) {
         pyr_fn(levels)<<<ctx->sm_count * 8, 256, 0, s>>>(ctx->d_call);
         VIO_CK(cudaGetLastError());
     }
@@ -466,7 +468,6 @@ vio_status launch(vio_ctx* ctx, int variant, const uint8_t* const* lev0, const i
         const uint64_t d = (uint64_t)(cell >> k);  // >= 2: cell is a multiple of 32, k <= 4
         hdr->cell_magic[k] = (uint32_t)(((1ull << 32) + d - 1) / d);
     }
-    const int B = 1 << (levels - 1);
     blocks[0] = 0;
     cells[0] = 0;
     for (int i = 0; i < n; ++i) {
@@ -476,12 +477,6 @@ vio_status launch(vio_ctx* ctx, int variant, const uint8_t* const* lev0, const i
         f.h = dims[i].h;
         f.gw = (f.w + cell - 1) / cell;
         f.gh = (f.h + cell - 1) / cell;
-        // pyramid CTAs cover 512 columns x 8B rows of level 0
-        f.pyr_bx = (f.w + 511) / 512;
-        f.pyr_magic = (uint32_t)(((1ull << 31) + f.pyr_bx - 1) / f.pyr_bx);
-        const int pyr_by = (f.h + 8 * B - 1) / (8 * B);
-        blocks[i + 1] = blocks[i] + (levels > 1 ? f.pyr_bx * pyr_by : 0);
-        cells[i + 1] = cells[i] + f.gw * f.gh;
         f.keys = ctx->d_keys + key_off[i];
         f.out = outs[i];
         f.lev[0] = const_cast<uint8_t*>(lev0[i]);
@@ -490,6 +485,8 @@ vio_status launch(vio_ctx* ctx, int variant, const uint8_t* const* lev0, const i
             f.src0 = up.src[i];
             f.src0_pitch = up.pitch[i];
         }
+        blocks[i + 1] = blocks[i] + pyr_plan(f, levels);
+        cells[i + 1] = cells[i] + f.gw * f.gh;
         if ((st = encode_map(ctx, &maps0[i], lev0[i], f.w, f.h, pitch0[i], kBoxW, v.th + 2 * v.radius + 6)) != VIO_OK)
             return st;
         for (int k = 1; k < levels; ++k) {
@@ -541,6 +538,7 @@ vio_status launch(vio_ctx* ctx, int variant, const uint8_t* const* lev0, const i
     const bool small = acc <= ctx->sm_count && blocks[n] <= 2 * ctx->sm_count &&
                        cells[n] <= kSmallDecodeCtas * 256 * 4;
 
+    pyramid = pyramid && blocks[n] > 0;
     VIO_CK(cudaMemcpyAsync(ctx->d_call, st_base, bytes, cudaMemcpyHostToDevice, s));
     VIO_CK(cudaEventRecord(ctx->ring_ev[slot], s));
     if (sweep) {
@@ -659,6 +657,46 @@ __global__ void selftest_wait_kernel(uint32_t* status, uint64_t limit_ns) {
     }
     __syncwarp();
     if (threadIdx.x == 0 && !mbar_wait_bounded(&bar, 0, limit_ns)) atomicOr(status, kStatusTimeout);
+}
+
+}  // namespace
+
+namespace {
+
+// Level-0 addresses of device frames: frames that TMA cannot address (a base or
+// pitch that is not a multiple of 16) get slots in the context's staging
+// buffer, which the pyramid kernel fills as it reads them (24 frames of odd
+// width took 24 copies, 100 us, before).
+struct Staging {
+    std::vector<const uint8_t*> lev0, src;
+    std::vector<int> pitch0, src_pitch;
+    bool any = false;
+    Upload upload() const { return any ? Upload{src.data(), src_pitch.data()} : Upload{}; }
+};
+
+vio_status plan_staging(vio_ctx* ctx, const uint8_t* const* frames, const vio_dims* dims, int n, Staging* out) {
+    out->lev0.assign(frames, frames + n);
+    out->src.assign(n, nullptr);
+    out->pitch0.resize(n);
+    out->src_pitch.assign(n, 0);
+    size_t need = 0;
+    std::vector<size_t> off(n, 0);
+    for (int i = 0; i < n; ++i) {
+        out->pitch0[i] = dims[i].pitch;
+        if (((uintptr_t)frames[i] & 15) || (dims[i].pitch & 15)) {
+            out->src[i] = frames[i];
+            out->src_pitch[i] = dims[i].pitch;
+            out->pitch0[i] = (int)align_up(dims[i].w, 16);
+            out->any = true;
+            off[i] = need;
+            need += align_up((size_t)out->pitch0[i] * dims[i].h, 256);
+        }
+    }
+    vio_status st;
+    if (out->any && (st = grow(ctx, (void**)&ctx->d_in, &ctx->in_cap, need, false)) != VIO_OK) return st;
+    for (int i = 0; i < n; ++i)
+        if (out->src[i]) out->lev0[i] = ctx->d_in + off[i];
+    return VIO_OK;
 }
 
 }  // namespace
@@ -888,33 +926,12 @@ vio_status vio_detect(vio_ctx* ctx, const uint8_t* const* frames, const vio_dims
     VIO_CK(cudaSetDevice(ctx->cfg.device));
     for (int i = 0; i < n; ++i)
         if (!frames[i] || !out_cells[i]) return fail(ctx, VIO_ERR_INVALID_ARG, "NULL frame or output pointer");
-    // frames that TMA cannot address directly are staged into aligned slots
-    std::vector<const uint8_t*> lev0(frames, frames + n);
-    std::vector<int> pitch0(n);
-    size_t need = 0;
-    std::vector<size_t> off(n, (size_t)-1);
-    for (int i = 0; i < n; ++i) {
-        pitch0[i] = dims[i].pitch;
-        if (((uintptr_t)frames[i] & 15) || (dims[i].pitch & 15)) {
-            off[i] = need;
-            need += align_up((size_t)align_up(dims[i].w, 16) * dims[i].h, 256);
-        }
-    }
-    if (need) {
-        if ((st = grow(ctx, (void**)&ctx->d_in, &ctx->in_cap, need, false)) != VIO_OK) return st;
-        for (int i = 0; i < n; ++i)
-            if (off[i] != (size_t)-1) {
-                const int p = (int)align_up(dims[i].w, 16);
-                VIO_CK(cudaMemcpy2DAsync(ctx->d_in + off[i], p, frames[i], dims[i].pitch, dims[i].w, dims[i].h,
-                                         cudaMemcpyDeviceToDevice, s));
-                lev0[i] = ctx->d_in + off[i];
-                pitch0[i] = p;
-            }
-    }
+    Staging stg;
+    if ((st = plan_staging(ctx, frames, dims, n, &stg)) != VIO_OK) return st;
     std::vector<int4*> outs(n);
     for (int i = 0; i < n; ++i) outs[i] = reinterpret_cast<int4*>(out_cells[i]);
-    return detect_impl(ctx, lev0.data(), pitch0.data(), dims, n, thresh, arc, cell, levels, outs.data(), out_counts,
-                       s);
+    return detect_impl(ctx, stg.lev0.data(), stg.pitch0.data(), dims, n, thresh, arc, cell, levels, outs.data(),
+                       out_counts, s, stg.upload());
 }
 
 vio_status vio_detect_sweep(vio_ctx* ctx, const uint8_t* const* frames, const vio_dims* dims, int n,
@@ -934,37 +951,16 @@ vio_status vio_detect_sweep(vio_ctx* ctx, const uint8_t* const* frames, const vi
         if (!out_cells[i]) return fail(ctx, VIO_ERR_INVALID_ARG, "NULL output pointer");
     for (int i = 0; i < n; ++i)
         if (!frames[i]) return fail(ctx, VIO_ERR_INVALID_ARG, "NULL frame pointer");
-    // frames that TMA cannot address directly are staged into aligned slots
-    std::vector<const uint8_t*> lev0(frames, frames + n);
-    std::vector<int> pitch0(n);
-    size_t need = 0;
-    std::vector<size_t> off(n, (size_t)-1);
-    for (int i = 0; i < n; ++i) {
-        pitch0[i] = dims[i].pitch;
-        if (((uintptr_t)frames[i] & 15) || (dims[i].pitch & 15)) {
-            off[i] = need;
-            need += align_up((size_t)align_up(dims[i].w, 16) * dims[i].h, 256);
-        }
-    }
-    if (need) {
-        if ((st = grow(ctx, (void**)&ctx->d_in, &ctx->in_cap, need, false)) != VIO_OK) return st;
-        for (int i = 0; i < n; ++i)
-            if (off[i] != (size_t)-1) {
-                const int p = (int)align_up(dims[i].w, 16);
-                VIO_CK(cudaMemcpy2DAsync(ctx->d_in + off[i], p, frames[i], dims[i].pitch, dims[i].w, dims[i].h,
-                                         cudaMemcpyDeviceToDevice, s));
-                lev0[i] = ctx->d_in + off[i];
-                pitch0[i] = p;
-            }
-    }
+    Staging stg;
+    if ((st = plan_staging(ctx, frames, dims, n, &stg)) != VIO_OK) return st;
     int vi = ctx->pinned_variant >= 0 ? ctx->pinned_variant : first_variant(ctx->cfg.nms_radius);
     if (ctx->pinned_variant < 0 && ctx->cfg.autotune) {
         const ShapeKey key = shape_key(dims, n, cell, levels);
         if (!ctx->tuned.count(key)) {
             std::vector<int4*> outs0(n);
             for (int i = 0; i < n; ++i) outs0[i] = reinterpret_cast<int4*>(out_cells[i]);
-            if ((st = autotune(ctx, key, lev0.data(), pitch0.data(), dims, n, thresholds[0], arc_lens[0], cell,
-                               levels, outs0.data(), out_counts, s)) != VIO_OK)
+            if ((st = autotune(ctx, key, stg.lev0.data(), stg.pitch0.data(), dims, n, thresholds[0], arc_lens[0],
+                               cell, levels, outs0.data(), out_counts, s, stg.upload())) != VIO_OK)
                 return st;
         }
         vi = ctx->tuned[key].variant;
@@ -998,8 +994,8 @@ vio_status vio_detect_sweep(vio_ctx* ctx, const uint8_t* const* frames, const vi
                 for (int i = 0; i < n; ++i) outs[(size_t)j * n + i] = reinterpret_cast<int4*>(out_cells[(size_t)p * n + i]);
             }
             sp.outs = outs.data();
-            if ((st = launch(ctx, v0, lev0.data(), pitch0.data(), dims, n, sp.thresh[0], sp.arc[0], cell, levels,
-                             outs.data(), nullptr, s, g0 == 0, {}, &sp)) != VIO_OK)
+            if ((st = launch(ctx, v0, stg.lev0.data(), stg.pitch0.data(), dims, n, sp.thresh[0], sp.arc[0], cell, levels,
+                             outs.data(), nullptr, s, g0 == 0, stg.upload(), &sp)) != VIO_OK)
                 return st;
         }
         return VIO_OK;
@@ -1008,8 +1004,9 @@ vio_status vio_detect_sweep(vio_ctx* ctx, const uint8_t* const* frames, const vi
     std::vector<int4*> outs(n);
     for (int p = 0; p < n_params; ++p) {
         for (int i = 0; i < n; ++i) outs[i] = reinterpret_cast<int4*>(out_cells[(size_t)p * n + i]);
-        if ((st = launch(ctx, vi, lev0.data(), pitch0.data(), dims, n, thresholds[p], arc_lens[p], cell, levels,
-                         outs.data(), out_counts ? out_counts + (size_t)p * n : nullptr, s, p == 0)) != VIO_OK)
+        if ((st = launch(ctx, vi, stg.lev0.data(), stg.pitch0.data(), dims, n, thresholds[p], arc_lens[p], cell, levels,
+                         outs.data(), out_counts ? out_counts + (size_t)p * n : nullptr, s, p == 0,
+                         stg.upload())) != VIO_OK)
             return st;
     }
     return VIO_OK;

@@ -224,13 +224,10 @@ extern "C" vio_status vio_detect_noalloc(const uint8_t* frame, vio_dims d, int t
         const uint64_t dv = (uint64_t)(cell >> k);
         hdr->cell_magic[k] = (uint32_t)(((1ull << 32) + dv - 1) / dv);
     }
-    const int B = 1 << (levels - 1);
     fd->w = d.w;
     fd->h = d.h;
     fd->gw = gw;
     fd->gh = gh;
-    fd->pyr_bx = (d.w + 511) / 512;
-    fd->pyr_magic = (uint32_t)(((1ull << 31) + fd->pyr_bx - 1) / fd->pyr_bx);
     fd->keys = keys;
     fd->out = reinterpret_cast<int4*>(out_cells);
     fd->lev[0] = const_cast<uint8_t*>(frame);
@@ -242,7 +239,7 @@ extern "C" vio_status vio_detect_noalloc(const uint8_t* frame, vio_dims d, int t
         if (!encode(&mapk[k - 1], fd->lev[k], d.w >> k, d.h >> k, lev_pitch[k])) return VIO_ERR_CUDA;
     }
     blocks[0] = 0;
-    blocks[1] = levels > 1 ? fd->pyr_bx * ((d.h + 8 * B - 1) / (8 * B)) : 0;
+    blocks[1] = pyr_plan(*fd, levels);
     cells[0] = 0;
     cells[1] = gw * gh;
     int acc = 0;

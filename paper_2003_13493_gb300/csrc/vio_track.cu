@@ -19,6 +19,7 @@ using PyrFn = void (*)(const uint8_t*);
 
 PyrFn track_pyr_fn(int levels) {
     switch (levels) {
+        case 1: return pyramid_kernel<1>;
         case 2: return pyramid_kernel<2>;
         case 3: return pyramid_kernel<3>;
         case 4: return pyramid_kernel<4>;
@@ -170,7 +171,6 @@ vio_status track_impl(vio_ctx* ctx, const uint8_t* const* prev, const uint8_t* c
     hdr->off_fds = (uint32_t)off_fds;
     hdr->off_blocks = (uint32_t)off_blocks;
     hdr->off_maps0 = hdr->off_mapsk = hdr->off_tiles = hdr->off_cells = (uint32_t)off_blocks;
-    const int B = 1 << (L - 1);
     blocks[0] = 0;
     for (int f = 0; f < nf; ++f) {
         const vio_dims& d = dims[f >> 1];
@@ -178,19 +178,17 @@ vio_status track_impl(vio_ctx* ctx, const uint8_t* const* prev, const uint8_t* c
         FrameDesc& fd = fds[f];
         fd.w = d.w;
         fd.h = d.h;
-        fd.pyr_bx = (d.w + 511) / 512;
-        fd.pyr_magic = (uint32_t)(((1ull << 31) + fd.pyr_bx - 1) / fd.pyr_bx);
-        const int pyr_by = (d.h + 8 * B - 1) / (8 * B);
-        blocks[f + 1] = blocks[f] + (L > 1 ? fd.pyr_bx * pyr_by : 0);
         if (in_off[f] != (size_t)-1) {
-            const int pp = (int)align_up(d.w, 16);
-            VIO_CK(cudaMemcpy2DAsync(T.d_in + in_off[f], pp, src, d.pitch, d.w, d.h, cudaMemcpyDeviceToDevice, s));
+            // copied by the pyramid kernel as it reads it
+            fd.src0 = src;
+            fd.src0_pitch = d.pitch;
             fd.lev[0] = T.d_in + in_off[f];
-            fd.pitch[0] = pp;
+            fd.pitch[0] = (int)align_up(d.w, 16);
         } else {
             fd.lev[0] = const_cast<uint8_t*>(src);
             fd.pitch[0] = d.pitch;
         }
+        blocks[f + 1] = blocks[f] + pyr_plan(fd, L);
         for (int k = 1; k < L; ++k) {
             fd.lev[k] = T.d_pyr + lev_off[f * kMaxLevels + k];
             fd.pitch[k] = lev_pitch[f * kMaxLevels + k];
@@ -219,7 +217,7 @@ vio_status track_impl(vio_ctx* ctx, const uint8_t* const* prev, const uint8_t* c
     VIO_CK(cudaEventRecord(T.stage_ev, s));
     // the kernel strides over its grid: a few frames' blocks need no more than one CTA per SM
     const int pyr_grid = blocks[nf] <= 2 * ctx->sm_count ? ctx->sm_count : ctx->sm_count * 8;
-    if (L > 1) track_pyr_fn(L)<<<pyr_grid, 256, 0, s>>>(T.d_call);
+    if (blocks[nf] > 0) track_pyr_fn(L)<<<pyr_grid, 256, 0, s>>>(T.d_call);
     VIO_CK(cudaGetLastError());
     const int grid = (int)((total + kTrackWarps - 1) / kTrackWarps);
     track_kernel<<<grid, kTrackWarps * 32, 0, s>>>(T.d_call, (uint32_t)off_track);
