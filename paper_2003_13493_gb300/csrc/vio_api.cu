@@ -378,12 +378,24 @@ vio_status enqueue_sweep(vio_ctx* ctx, int levels, cudaStream_t s, bool pyramid,
         VIO_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fast_sweep_kernel<kSweepTH>, kThreads, smem));
         ctx->grid_sweep = std::max(1, occ) * ctx->sm_count;
     }
-    fast_sweep_kernel<kSweepTH><<<ctx->grid_sweep, kThreads, smem, s>>>(ctx->d_call, d_sw, ctx->d_counter,
-                                                                      ctx->d_status);
-    VIO_CK(cudaGetLastError());
+    // programmatic dependents, as in enqueue_kernels
+    cudaLaunchAttribute pdl[1];
+    pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    pdl[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(ctx->grid_sweep);
+    lc.blockDim = dim3(kThreads);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = s;
+    lc.attrs = pdl;
+    lc.numAttrs = 1;
+    VIO_CK(cudaLaunchKernelEx(&lc, fast_sweep_kernel<kSweepTH>, (const uint8_t*)ctx->d_call, d_sw, ctx->d_counter,
+                              ctx->d_status));
     if (prof) VIO_CK(cudaEventRecord(ctx->stage_ev[2], s));
-    sweep_decode_kernel<<<ctx->sm_count * 4, 256, 0, s>>>(ctx->d_call, d_sw, ctx->d_counter);
-    VIO_CK(cudaGetLastError());
+    lc.gridDim = dim3(ctx->sm_count * 4);
+    lc.blockDim = dim3(256);
+    lc.dynamicSmemBytes = 0;
+    VIO_CK(cudaLaunchKernelEx(&lc, sweep_decode_kernel, (const uint8_t*)ctx->d_call, d_sw, ctx->d_counter));
     if (prof) VIO_CK(cudaEventRecord(ctx->stage_ev[3], s));
     return VIO_OK;
 }

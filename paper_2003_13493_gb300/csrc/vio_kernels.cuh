@@ -1107,12 +1107,12 @@ __global__ void __launch_bounds__(kThreads, 4) fast_nms_cell_kernel(const uint8_
 // (warp-aggregated; the fused kernel zeroed the counts).
 // ---------------------------------------------------------------------------
 static __global__ void __launch_bounds__(256) decode_kernel(const uint8_t* __restrict__ call, int32_t* __restrict__ counter) {
-    // the cell keys are final once the detect kernel before this one has
-    // completed (it may still be running: programmatic dependent launch)
-    griddep_wait();
     const CallView cv(call);
     const int nf = cv.h->n_frames, total = cv.h->n_cells;
     int32_t* counts = cv.h->counts;
+    uint32_t* status = cv.h->status;
+    const uint32_t magic = cv.h->cell_magic[0];
+    const int levels = cv.h->levels;
     const int lane = threadIdx.x & 31;
     // the cell prefix sums in shared memory when they fit (see pyramid_kernel)
     __shared__ int32_t cells_sh[kPrefixCache];
@@ -1120,33 +1120,47 @@ static __global__ void __launch_bounds__(256) decode_kernel(const uint8_t* __res
     if (nf < kPrefixCache)
         for (int j = threadIdx.x; j <= nf; j += blockDim.x) cells_sh[j] = cv.cells[j];
     __syncthreads();
+    // the cell keys are final once the detect kernel before this one has
+    // completed; it may still be running (programmatic dependent launch), so
+    // the cell's frame, which the call block holds since before, is found first
+    bool keys_final = false;
     for (int base = blockIdx.x * blockDim.x; base < total; base += gridDim.x * blockDim.x) {
         const int i = base + threadIdx.x;
-        int f = -1;
-        bool hit = false;
+        int f = -1, c = 0, w = 1, h = 0, gw = 0;
+        uint64_t* kp = nullptr;
+        int4* out = nullptr;
         if (i < total) {
             f = upper_index(cells, nf, i);
             const FrameDesc& fd = cv.fds[f];
-            const int c = i - cells[f];
-            const uint64_t key = fd.keys[c];
+            c = i - cells[f];
+            w = fd.w;
+            h = fd.h;
+            gw = fd.gw;
+            kp = fd.keys + c;
+            out = fd.out + c;
+        }
+        if (!keys_final) griddep_wait();
+        keys_final = true;
+        bool hit = false;
+        if (i < total) {
+            const uint64_t key = *kp;
             int4 rec = make_int4(-1, -1, -1, 0);
             if (key != 0) {
                 const uint32_t lin = 0xFFFFFFFFu - (uint32_t)key;
                 const int k = (int)(lin >> 28);
                 const uint32_t idx = lin & 0x0FFFFFFFu;
-                const uint32_t wk = (uint32_t)(fd.w >> k);
+                const uint32_t wk = (uint32_t)(w >> k);
                 const int y = (int)(idx / wk), x = (int)(idx - (uint32_t)y * wk);
                 rec = make_int4(x << k, y << k, k, (int)(key >> 32));
-                fd.keys[c] = 0;
+                *kp = 0;
                 hit = true;
                 // consistency of the packed key with the cell it was folded into
-                const uint32_t magic = cv.h->cell_magic[0];
-                if (cv.h->status && (k >= cv.h->levels || rec.x >= fd.w || rec.y >= fd.h ||
-                                     __umulhi((uint32_t)rec.y, magic) * (uint32_t)fd.gw +
-                                             __umulhi((uint32_t)rec.x, magic) != (uint32_t)c))
-                    atomicOr(cv.h->status, kStatusBadKey);
+                if (status && (k >= levels || rec.x >= w || rec.y >= h ||
+                               __umulhi((uint32_t)rec.y, magic) * (uint32_t)gw + __umulhi((uint32_t)rec.x, magic) !=
+                                   (uint32_t)c))
+                    atomicOr(status, kStatusBadKey);
             }
-            fd.out[c] = rec;
+            *out = rec;
         }
         if (counts) {
             // lanes of one frame add their hits with one atomic
@@ -1161,6 +1175,7 @@ static __global__ void __launch_bounds__(256) decode_kernel(const uint8_t* __res
             }
         }
     }
+    if (!keys_final) griddep_wait();
     if (blockIdx.x == 0 && threadIdx.x == 0) *counter = 0;
 }
 

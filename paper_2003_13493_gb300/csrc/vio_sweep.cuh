@@ -102,6 +102,7 @@ __global__ void __launch_bounds__(kThreads, 3) fast_sweep_kernel(const uint8_t* 
         for (int i = tid; i < n_tiles; i += kThreads) tiles_sh[i] = cv.tiles[i];
     __syncthreads();
 
+    griddep_launch_dependents();
     if (warp == kConsumers / 32) {
         produce_tiles<TH, 1>(cv, cached ? tiles_sh : cv.tiles, counter, status, info, full_bar, empty_bar, smem, lane);
         return;
@@ -339,6 +340,7 @@ static __global__ void __launch_bounds__(256) sweep_decode_kernel(const uint8_t*
     if (nf < kPrefixCache)
         for (int j = threadIdx.x; j <= nf; j += blockDim.x) cells_sh[j] = cv.cells[j];
     __syncthreads();
+    griddep_wait();  // the keys are final once the sweep kernel has completed
     for (int base = blockIdx.x * blockDim.x; base < total; base += gridDim.x * blockDim.x) {
         const int i = base + threadIdx.x;
         int g = -1;  // (setting, frame) group of this thread
