@@ -18,6 +18,7 @@
 #include "vio_ctx.h"
 #include "vio_kernels.cuh"
 #include "vio_sweep.cuh"
+#include "vio_tiles.cuh"
 
 using namespace vio;
 
@@ -637,6 +638,12 @@ vio_status autotune(vio_ctx* ctx, const ShapeKey& key, const uint8_t* const* lev
 vio_status detect_impl(vio_ctx* ctx, const uint8_t* const* lev0, const int* pitch0, const vio_dims* dims, int n,
                        int thresh, int arc, int cell, int levels, int4* const* outs, int32_t* counts,
                        cudaStream_t s, Upload up = {}) {
+    if (!up.src) {
+        bool done = false;
+        const vio_status st = vio::detect_tiles(ctx, lev0, pitch0, dims, n, thresh, arc, cell ? cell : 32, levels, outs,
+                                                counts, s, &done);
+        if (st != VIO_OK || done) return st;
+    }
     int vi = ctx->pinned_variant;
     int ctas = ctx->pinned_ctas;
     int c = cell ? cell : 32;
@@ -859,6 +866,7 @@ vio_status vio_create(vio_ctx** out, const vio_config* cfg_in) {
     vio_ctx* ctx = new vio_ctx();
     ctx->cfg = cfg;
     ctx->sm_count = prop.multiProcessorCount;
+    ctx->default_variant = first_variant(cfg.nms_radius);
     ctx->call_cap = call_block_cap(cfg.max_frames);
     cudaDriverEntryPointQueryResult q;
     void* fnp = nullptr;
@@ -873,8 +881,11 @@ vio_status vio_create(vio_ctx** out, const vio_config* cfg_in) {
         return s;
     };
     if (cudaMalloc(&ctx->d_call, ctx->call_cap) != cudaSuccess) return cleanup(VIO_ERR_OOM);
-    if (cudaMalloc(&ctx->d_counter, sizeof(int32_t) * 4) != cudaSuccess) return cleanup(VIO_ERR_OOM);
-    if (cudaMemset(ctx->d_counter, 0, sizeof(int32_t) * 4) != cudaSuccess) return cleanup(VIO_ERR_CUDA);
+    constexpr size_t counter_bytes = 16 + (sizeof(uint64_t) + sizeof(int32_t)) * kTileCap[1];
+    if (cudaMalloc(&ctx->d_counter, counter_bytes) != cudaSuccess) return cleanup(VIO_ERR_OOM);
+    if (cudaMemset(ctx->d_counter, 0, counter_bytes) != cudaSuccess) return cleanup(VIO_ERR_CUDA);
+    ctx->d_sums = reinterpret_cast<uint64_t*>(ctx->d_counter + 4);
+    ctx->d_done = reinterpret_cast<int32_t*>(ctx->d_sums + kTileCap[1]);
     if (cudaHostAlloc(&ctx->h_status, 64, cudaHostAllocMapped) != cudaSuccess) return cleanup(VIO_ERR_OOM);
     *ctx->h_status = 0;
     if (cudaHostGetDevicePointer((void**)&ctx->d_status, ctx->h_status, 0) != cudaSuccess)
@@ -938,6 +949,14 @@ vio_status vio_detect(vio_ctx* ctx, const uint8_t* const* frames, const vio_dims
     VIO_CK(cudaSetDevice(ctx->cfg.device));
     for (int i = 0; i < n; ++i)
         if (!frames[i] || !out_cells[i]) return fail(ctx, VIO_ERR_INVALID_ARG, "NULL frame or output pointer");
+    {
+        std::array<int, kTileCap[1]> pitch;
+        for (int i = 0; i < n && i < kTileCap[1]; ++i) pitch[i] = dims[i].pitch;
+        bool done = false;
+        st = vio::detect_tiles(ctx, frames, pitch.data(), dims, n, thresh, arc, cell ? cell : 32, levels,
+                               reinterpret_cast<int4* const*>(out_cells), out_counts, s, &done);
+        if (st != VIO_OK || done) return st;
+    }
     Staging stg;
     if ((st = plan_staging(ctx, frames, dims, n, &stg)) != VIO_OK) return st;
     std::vector<int4*> outs(n);

@@ -106,6 +106,9 @@ struct vio_ctx {
     // resident device buffers
     uint8_t* d_call = nullptr;          // the current call block
     int32_t* d_counter = nullptr;       // work-item counter of the fused kernel
+    // in the same allocation, zero when idle (see TileCall)
+    uint64_t* d_sums = nullptr;
+    int32_t* d_done = nullptr;
     uint64_t* d_keys = nullptr;         // packed cell keys, zero when idle
     size_t keys_cap = 0;
     uint8_t* d_pyr = nullptr;           // pyramid levels 1..L-1 of every frame
@@ -137,6 +140,8 @@ struct vio_ctx {
     cudaGraphExec_t graphs[8][vio::kMaxLevels + 1][2][vio::kMaxCtasPerSm + 1] = {};
     int occ_fused[8] = {};                 // CTAs per SM that fit, per variant
     int grid_sweep = 0;
+    bool tile_ready[2] = {};               // attributes of the two forms of tile_detect_kernel are set
+    int default_variant = 0;               // first variant of the context's NMS radius
     struct TuneChoice {
         int variant, ctas, cell;
     };
@@ -226,6 +231,11 @@ namespace vio {
 // nullptr.  Arguments are checked by the caller.
 vio_status detect_from_host(vio_ctx* ctx, const uint8_t* const* host_frames, const vio_dims* dims, int n, int thresh,
                             int arc, int cell, int levels, int4* const* outs, int32_t* d_counts, cudaStream_t s);
+// Detects with tile_detect_kernel (vio_tiles.cuh) when the call is one that it
+// takes, and sets *done then.  Frames of any alignment, in device memory.
+vio_status detect_tiles(vio_ctx* ctx, const uint8_t* const* lev0, const int* pitch0, const vio_dims* dims, int n,
+                        int thresh, int arc, int cell, int levels, int4* const* outs, int32_t* counts, cudaStream_t s,
+                        bool* done);
 // Device address of pinned host memory, else nullptr.
 const void* host_device_alias(const void* host);
 }  // namespace vio

@@ -550,6 +550,28 @@ struct ItemInfo {
     uint64_t* keys;
 };
 
+// The constants of a tile whose x0, y0, wk and hk are set: score column 0 is
+// level x = x0 - 4 and box column 0 is (x0 - 8) & ~15; score row r is level
+// y = y0 - R + r; testable pixels are 3 <= x < Wk - 3, 3 <= y < Hk - 3; the NMS
+// reads score columns 4 - R .. 123 + R only.
+template <int TH, int R>
+__device__ __forceinline__ void tile_constants(ItemInfo& in) {
+    in.xoff = in.x0 - 4 - ((in.x0 - 8) & ~15);
+    in.row_lo = max(0, 3 - in.y0 + R);
+    in.row_hi = min(TileGeom<TH, R>::SR, in.hk - 3 - in.y0 + R);
+    in.xlo = max(4 - R, 7 - in.x0);
+    in.xhi = min(124 + R, in.wk + 1 - in.x0);
+}
+
+// Bit 7 of byte j set when xlo <= 4 lane + j < xhi: byte j of cols4 + (128 - x)
+// reaches bit 7 exactly when 4 lane + j >= x (all values below 256: no carries
+// between bytes).
+__device__ __forceinline__ uint32_t kept_columns(const ItemInfo& in, int lane) {
+    const uint32_t cols4 = (uint32_t)(4 * lane) * 0x01010101u + 0x03020100u;
+    return (cols4 + (uint32_t)(0x80 - in.xlo) * 0x01010101u) & ~(cols4 + (uint32_t)(0x80 - in.xhi) * 0x01010101u) &
+           0x80808080u;
+}
+
 // upper_index by a whole warp (all lanes call it with the same arguments):
 // 32 entries per step, so 1024 entries take two dependent loads instead of ten.
 __device__ __forceinline__ int upper_index_warp(const int32_t* a, int n, int v, int lane) {
@@ -829,16 +851,8 @@ __device__ __forceinline__ void produce_tiles(const CallView& cv, const int32_t*
             const int ty = ti / ntx;
             in.x0 = (ti - ty * ntx) * G::TW;
             in.y0 = ty * TH;
-            // per-item constants, computed once here instead of by every
-            // consumer warp: score column 0 is level x = x0 - 4 and box column
-            // 0 is (x0 - 8) & ~15; score row r is level y = y0 - R + r; testable
-            // pixels are 3 <= x < Wk - 3, 3 <= y < Hk - 3; the NMS reads score
-            // columns 4 - R .. 123 + R only
-            in.xoff = in.x0 - 4 - ((in.x0 - 8) & ~15);
-            in.row_lo = max(0, 3 - in.y0 + R);
-            in.row_hi = min(G::SR, in.hk - 3 - in.y0 + R);
-            in.xlo = max(4 - R, 7 - in.x0);
-            in.xhi = min(124 + R, in.wk + 1 - in.x0);
+            // computed once here instead of by every consumer warp
+            tile_constants<TH, R>(in);
             map = in.level == 0 ? &cv.maps0[f] : &cv.mapsk[f * (kMaxLevels - 1) + in.level - 1];
             if (lane == 0) fence_tensormap_acquire(map);
             if (!pyramid_done && (in.level > 0 || uploaded)) {
@@ -893,6 +907,132 @@ __device__ __forceinline__ int nms_ring_pass(uint16_t* queue, int n, const uint1
         np += __popc(bm);
     }
     return np;
+}
+
+// Full segment test of a warp's queue (raw walk codes); the corners, as score
+// indices, are compacted in place.  Returns how many.
+template <int MODE, int TH, int R>
+__device__ __forceinline__ int full_test(const uint8_t* img_base, uint16_t* queue, int total, int warp, int lane,
+                                         uint32_t lt_mask, int thresh, int n_arc, uint32_t* status) {
+    using G = TileGeom<TH, R>;
+    int ncorner = 0;
+    for (int e0 = 0; e0 < total; e0 += 32) {
+        const int e = e0 + lane;
+        uint32_t s = 0;
+        int idx = 0;
+        if (e < total && vio_guard(e < G::QCAP, status)) {
+            idx = walk_code_index(queue[e], 2 * G::PPW * warp);
+            // box offset of score-region pixel (idx >> 7, idx & 127); the
+            // score is taken below, on the compacted corners only
+            if (vio_guard(idx < G::SR * G::SW, status))
+                s = eval_corner<MODE, G::BW, false>(img_base + idx + 16 * (idx >> 7), thresh, n_arc);
+        }
+        const uint32_t cm = __ballot_sync(0xFFFFFFFFu, s != 0);
+        if (s) queue[ncorner + __popc(cm & lt_mask)] = (uint16_t)idx;
+        ncorner += __popc(cm);
+    }
+    return ncorner;
+}
+
+// Scores of the corners queue[0, ncorner) into the score tile.
+template <int MODE, int TH, int R>
+__device__ __forceinline__ void score_corners(const uint8_t* img_base, const uint16_t* queue, int ncorner, int lane,
+                                              int thresh, int n_arc, uint16_t* sc) {
+    using G = TileGeom<TH, R>;
+    for (int e = lane; e < ncorner; e += 32) {
+        const int idx = queue[e];
+        const uint8_t* p = img_base + idx + 16 * (idx >> 7);
+        // MT of a known corner needs no segment test: the largest window
+        // minimum alone (see eval_corner)
+        sc[idx] = (uint16_t)(MODE == 0   ? sad_b<G::BW>(p)
+                             : MODE == 2 ? mt_of_corner<G::BW>(p, n_arc)
+                                         : eval_corner<MODE, G::BW, true>(p, thresh, n_arc));
+    }
+}
+
+// NMS on the corners queue[0, ncorner), cell maximum by a 64-bit max reduction
+// per survivor.  A window wider than 3x3 is tested ring by ring: the 8
+// nearest neighbours of every corner first, which suppress most
+// corners, then each further ring on the corners that passed the
+// rings inside it (compacted to the front of the queue).
+template <int TH, int R>
+__device__ __forceinline__ void nms_corners(uint16_t* queue, int ncorner, const uint16_t* sc, int lane,
+                                            uint32_t lt_mask, const ItemInfo& in, uint32_t* status) {
+    using G = TileGeom<TH, R>;
+    const int k = in.level, Wk = in.wk, x0 = in.x0, y0 = in.y0;
+    const uint32_t magic = in.magic;
+    int nnms = ncorner;
+    if constexpr (R > 1) {
+        int npass = 0;
+        for (int e0 = 0; e0 < ncorner; e0 += 32) {
+            const int e = e0 + lane;
+            int idx = 0;
+            bool ok = false;
+            if (e < ncorner) {
+                idx = queue[e];
+                const int sr = idx >> 7, scx = idx & 127;
+                if (scx >= 4 && scx < 4 + G::TW && sr >= R && sr < R + TH) {
+                    const uint16_t* q = sc + idx;
+                    const uint32_t s = q[0];
+                    ok = true;
+#pragma unroll
+                    for (int dy = -1; dy <= 1; ++dy)
+#pragma unroll
+                        for (int dx = -1; dx <= 1; ++dx)
+                            if (dy != 0 || dx != 0) ok &= s >= q[dy * G::SW + dx];
+                }
+            }
+            const uint32_t bm = __ballot_sync(0xFFFFFFFFu, ok);
+            if (ok) queue[npass + __popc(bm & lt_mask)] = (uint16_t)idx;
+            npass += __popc(bm);
+        }
+        nnms = npass;
+        if constexpr (R > 2) nnms = nms_ring_pass<2, G::SW>(queue, nnms, sc, lane, lt_mask);
+        if constexpr (R > 3) nnms = nms_ring_pass<3, G::SW>(queue, nnms, sc, lane, lt_mask);
+    }
+    for (int e0 = 0; e0 < nnms; e0 += 32) {
+        const int e = e0 + lane;
+        uint32_t cell_id = 0xFFFFFFFFu;
+        uint32_t hi = 0, lo = 0;
+        if (e < nnms) {
+            const int idx = queue[e];
+            const int sr = idx >> 7, scx = idx & 127;
+            // (with R > 1 the first pass kept corners inside the tile only)
+            const bool inside = R > 1 || (scx >= 4 && scx < 4 + G::TW && sr >= R && sr < R + TH);
+            if (inside) {
+                // (2R+1) x (2R+1) neighbourhood: keep when >= every neighbour
+                // (for R > 1 the outermost ring; the passes above did the rest)
+                const uint16_t* q = sc + idx;
+                const uint32_t s = q[0];
+                bool keep = true;
+                if constexpr (R == 1) {
+                    // (this loop form, not ring_max<1>: the MT kernel is
+                    // 5 % slower with the latter)
+#pragma unroll
+                    for (int dy = -1; dy <= 1; ++dy)
+#pragma unroll
+                        for (int dx = -1; dx <= 1; ++dx)
+                            if (dy != 0 || dx != 0) keep &= s >= q[dy * G::SW + dx];
+                } else {
+                    keep = ring_max<R, G::SW>(q, s);
+                }
+                if (keep) {
+                    const uint32_t x = (uint32_t)(x0 - 4 + scx), y = (uint32_t)(y0 - R + sr);
+                    const uint32_t cx = __umulhi(x, magic), cy = __umulhi(y, magic);
+                    if (vio_guard(cx < (uint32_t)in.gw && cy < (uint32_t)in.gh, status)) {
+                        cell_id = cy * (uint32_t)in.gw + cx;
+                        hi = s;
+                        lo = 0xFFFFFFFFu - (((uint32_t)k << 28) | (y * (uint32_t)Wk + x));
+                    }
+                }
+            }
+        }
+        // each survivor folds its key into the cell's (a warp-wide max
+        // for survivors sharing a cell first was 2.6 % slower: its votes,
+        // shuffle and reductions form one long dependent chain)
+        if (hi != 0) red_max_u64(reinterpret_cast<unsigned long long*>(&in.keys[cell_id]),
+                                 ((unsigned long long)hi << 32) | lo);
+    }
 }
 
 template <int TH, int MODE, int R = 1>
@@ -960,55 +1100,22 @@ __global__ void __launch_bounds__(kThreads, 4) fast_nms_cell_kernel(const uint8_
         const ItemInfo in = info[b];
         if (in.id >= n_items) break;
         const uint8_t* img = smem + G::IMG_OFF + b * G::BOXA;
-        const int k = in.level, Wk = in.wk, x0 = in.x0, y0 = in.y0;
-        const uint32_t magic = in.magic;
         const int xoff = in.xoff;
 
-        // 2. coarse test + compaction.  Testable pixels: 3 <= x < Wk-3, 3 <= y < Hk-3.
-        int total;
-        {
-            // score row r is level y = y0 - R + r; score column c is level x = x0 - 4 + c
-            const int row_lo = in.row_lo, row_hi = in.row_hi;
-            // vm: bit 7 of byte j set when xlo <= 4 lane + j < xhi; byte j of
-            // cols4 + (128 - x) reaches bit 7 exactly when 4 lane + j >= x
-            // (all values below 256: no carries between bytes)
-            const uint32_t cols4 = (uint32_t)(4 * lane) * 0x01010101u + 0x03020100u;
-            const uint32_t vm = (cols4 + (uint32_t)(0x80 - in.xlo) * 0x01010101u) &
-                                ~(cols4 + (uint32_t)(0x80 - in.xhi) * 0x01010101u) & 0x80808080u;
-            const int xw = xoff / 4;
-            total = high_t ? coarse_and_compact<true, TH, R>(img, queue, xw, k7, n_arc, warp, lane, row_lo, row_hi, vm, status)
-                           : coarse_and_compact<false, TH, R>(img, queue, xw, k7, n_arc, warp, lane, row_lo, row_hi, vm, status);
-        }
+        // 2. coarse test + compaction
+        const uint32_t vm = kept_columns(in, lane);
+        const int total =
+            high_t ? coarse_and_compact<true, TH, R>(img, queue, xoff / 4, k7, n_arc, warp, lane, in.row_lo, in.row_hi,
+                                                     vm, status)
+                   : coarse_and_compact<false, TH, R>(img, queue, xoff / 4, k7, n_arc, warp, lane, in.row_lo,
+                                                      in.row_hi, vm, status);
         __syncwarp();
 
-        // 3. full test on this warp's queue; corners are compacted in place
-        int ncorner = 0;
+        // 3. full test on this warp's queue
         const uint8_t* img_base = img + 3 * G::BW + xoff;
-        for (int e0 = 0; e0 < total; e0 += 32) {
-            const int e = e0 + lane;
-            uint32_t s = 0;
-            int idx = 0;
-            if (e < total && vio_guard(e < G::QCAP, status)) {
-                idx = walk_code_index(queue[e], 2 * G::PPW * warp);
-                // box offset of score-region pixel (idx >> 7, idx & 127); the
-                // score is taken below, on the compacted corners only
-                if (vio_guard(idx < G::SR * G::SW, status))
-                    s = eval_corner<MODE, G::BW, false>(img_base + idx + 16 * (idx >> 7), thresh, n_arc);
-            }
-            const uint32_t cm = __ballot_sync(0xFFFFFFFFu, s != 0);
-            if (s) queue[ncorner + __popc(cm & lt_mask)] = (uint16_t)idx;
-            ncorner += __popc(cm);
-        }
+        const int ncorner = full_test<MODE, TH, R>(img_base, queue, total, warp, lane, lt_mask, thresh, n_arc, status);
         if (!own_rows_reset<TH, R>(nms_bar, t, sc, warp, lane, status)) return;
-        for (int e = lane; e < ncorner; e += 32) {
-            const int idx = queue[e];
-            const uint8_t* p = img_base + idx + 16 * (idx >> 7);
-            // MT of a known corner needs no segment test: the largest window
-            // minimum alone (see eval_corner)
-            sc[idx] = (uint16_t)(MODE == 0   ? sad_b<G::BW>(p)
-                                 : MODE == 2 ? mt_of_corner<G::BW>(p, n_arc)
-                                             : eval_corner<MODE, G::BW, true>(p, thresh, n_arc));
-        }
+        score_corners<MODE, TH, R>(img_base, queue, ncorner, lane, thresh, n_arc, sc);
         // this warp is done with the image buffer, and its scores are written
         __syncwarp();
         if (lane == 0) {
@@ -1018,87 +1125,29 @@ __global__ void __launch_bounds__(kThreads, 4) fast_nms_cell_kernel(const uint8_
         // the neighbours' scores of this tile are written
         if (!neighbours_wait(sc_bar, warp, G::WARPS, t & 1, lane, status)) return;
 
-        // 4. NMS on the corners, cell maximum by a 64-bit max reduction per
-        // survivor.  A window wider than 3x3 is tested ring by ring: the 8
-        // nearest neighbours of every corner first, which suppress most
-        // corners, then each further ring on the corners that passed the
-        // rings inside it (compacted to the front of the queue).
-        int nnms = ncorner;
-        if constexpr (R > 1) {
-            int npass = 0;
-            for (int e0 = 0; e0 < ncorner; e0 += 32) {
-                const int e = e0 + lane;
-                int idx = 0;
-                bool ok = false;
-                if (e < ncorner) {
-                    idx = queue[e];
-                    const int sr = idx >> 7, scx = idx & 127;
-                    if (scx >= 4 && scx < 4 + G::TW && sr >= R && sr < R + TH) {
-                        const uint16_t* q = sc + idx;
-                        const uint32_t s = q[0];
-                        ok = true;
-#pragma unroll
-                        for (int dy = -1; dy <= 1; ++dy)
-#pragma unroll
-                            for (int dx = -1; dx <= 1; ++dx)
-                                if (dy != 0 || dx != 0) ok &= s >= q[dy * G::SW + dx];
-                    }
-                }
-                const uint32_t bm = __ballot_sync(0xFFFFFFFFu, ok);
-                if (ok) queue[npass + __popc(bm & lt_mask)] = (uint16_t)idx;
-                npass += __popc(bm);
-            }
-            nnms = npass;
-            if constexpr (R > 2) nnms = nms_ring_pass<2, G::SW>(queue, nnms, sc, lane, lt_mask);
-            if constexpr (R > 3) nnms = nms_ring_pass<3, G::SW>(queue, nnms, sc, lane, lt_mask);
-        }
-        for (int e0 = 0; e0 < nnms; e0 += 32) {
-            const int e = e0 + lane;
-            uint32_t cell_id = 0xFFFFFFFFu;
-            uint32_t hi = 0, lo = 0;
-            if (e < nnms) {
-                const int idx = queue[e];
-                const int sr = idx >> 7, scx = idx & 127;
-                // (with R > 1 the first pass kept corners inside the tile only)
-                const bool inside = R > 1 || (scx >= 4 && scx < 4 + G::TW && sr >= R && sr < R + TH);
-                if (inside) {
-                    // (2R+1) x (2R+1) neighbourhood: keep when >= every neighbour
-                    // (for R > 1 the outermost ring; the passes above did the rest)
-                    const uint16_t* q = sc + idx;
-                    const uint32_t s = q[0];
-                    bool keep = true;
-                    if constexpr (R == 1) {
-                        // (this loop form, not ring_max<1>: the MT kernel is
-                        // 5 % slower with the latter)
-#pragma unroll
-                        for (int dy = -1; dy <= 1; ++dy)
-#pragma unroll
-                            for (int dx = -1; dx <= 1; ++dx)
-                                if (dy != 0 || dx != 0) keep &= s >= q[dy * G::SW + dx];
-                    } else {
-                        keep = ring_max<R, G::SW>(q, s);
-                    }
-                    if (keep) {
-                        const uint32_t x = (uint32_t)(x0 - 4 + scx), y = (uint32_t)(y0 - R + sr);
-                        const uint32_t cx = __umulhi(x, magic), cy = __umulhi(y, magic);
-                        if (vio_guard(cx < (uint32_t)in.gw && cy < (uint32_t)in.gh, status)) {
-                            cell_id = cy * (uint32_t)in.gw + cx;
-                            hi = s;
-                            lo = 0xFFFFFFFFu - (((uint32_t)k << 28) | (y * (uint32_t)Wk + x));
-                        }
-                    }
-                }
-            }
-            // each survivor folds its key into the cell's (a warp-wide max
-            // for survivors sharing a cell first was 2.6 % slower: its votes,
-            // shuffle and reductions form one long dependent chain)
-            if (hi != 0) red_max_u64(reinterpret_cast<unsigned long long*>(&in.keys[cell_id]),
-                                     ((unsigned long long)hi << 32) | lo);
-        }
+        // 4. NMS and cell maximum
+        nms_corners<TH, R>(queue, ncorner, sc, lane, lt_mask, in, status);
         // this warp's NMS reads of the score tile are done
         __syncwarp();
         if (lane == 0) mbar_arrive(&nms_bar[warp]);
     }
+}
+
+// The record of a non-empty cell key of cell c of a w x h frame (gw cells per
+// row); reports a key that does not lie in its cell.
+__device__ __forceinline__ int4 decode_key(uint64_t key, int c, int w, int h, int gw, int levels, uint32_t magic,
+                                           uint32_t* status) {
+    const uint32_t lin = 0xFFFFFFFFu - (uint32_t)key;
+    const int k = (int)(lin >> 28);
+    const uint32_t idx = lin & 0x0FFFFFFFu;
+    const uint32_t wk = (uint32_t)(w >> k);
+    const int y = (int)(idx / wk), x = (int)(idx - (uint32_t)y * wk);
+    const int4 rec = make_int4(x << k, y << k, k, (int)(key >> 32));
+    // consistency of the packed key with the cell it was folded into
+    if (status && (k >= levels || rec.x >= w || rec.y >= h ||
+                   __umulhi((uint32_t)rec.y, magic) * (uint32_t)gw + __umulhi((uint32_t)rec.x, magic) != (uint32_t)c))
+        atomicOr(status, kStatusBadKey);
+    return rec;
 }
 
 // ---------------------------------------------------------------------------
@@ -1146,19 +1195,9 @@ static __global__ void __launch_bounds__(256) decode_kernel(const uint8_t* __res
             const uint64_t key = *kp;
             int4 rec = make_int4(-1, -1, -1, 0);
             if (key != 0) {
-                const uint32_t lin = 0xFFFFFFFFu - (uint32_t)key;
-                const int k = (int)(lin >> 28);
-                const uint32_t idx = lin & 0x0FFFFFFFu;
-                const uint32_t wk = (uint32_t)(w >> k);
-                const int y = (int)(idx / wk), x = (int)(idx - (uint32_t)y * wk);
-                rec = make_int4(x << k, y << k, k, (int)(key >> 32));
+                rec = decode_key(key, c, w, h, gw, levels, magic, status);
                 *kp = 0;
                 hit = true;
-                // consistency of the packed key with the cell it was folded into
-                if (status && (k >= levels || rec.x >= w || rec.y >= h ||
-                               __umulhi((uint32_t)rec.y, magic) * (uint32_t)gw + __umulhi((uint32_t)rec.x, magic) !=
-                                   (uint32_t)c))
-                    atomicOr(status, kStatusBadKey);
             }
             *out = rec;
         }

@@ -169,9 +169,7 @@ __global__ void __launch_bounds__(kThreads, 3) fast_sweep_kernel(const uint8_t* 
         {
             // the producer's per-item rows and columns (NMS radius 1)
             const int row_lo = in.row_lo, row_hi = in.row_hi;
-            const uint32_t cols4 = (uint32_t)(4 * lane) * 0x01010101u + 0x03020100u;
-            const uint32_t vm = (cols4 + (uint32_t)(0x80 - in.xlo) * 0x01010101u) &
-                                ~(cols4 + (uint32_t)(0x80 - in.xhi) * 0x01010101u) & 0x80808080u;
+            const uint32_t vm = kept_columns(in, lane);
             const int xw = xoff / 4;
             // levels >= 1: the run of even circle points that the shortest
             // arc needs; level 0, where few pixels pass at all: two compass points
@@ -354,19 +352,9 @@ static __global__ void __launch_bounds__(256) sweep_decode_kernel(const uint8_t*
             const uint64_t key = *kp;
             int4 rec = make_int4(-1, -1, -1, 0);
             if (key != 0) {
-                const uint32_t lin = 0xFFFFFFFFu - (uint32_t)key;
-                const int k = (int)(lin >> 28);
-                const uint32_t idx = lin & 0x0FFFFFFFu;
-                const uint32_t wk = (uint32_t)(fd.w >> k);
-                const int y = (int)(idx / wk), x = (int)(idx - (uint32_t)y * wk);
-                rec = make_int4(x << k, y << k, k, (int)(key >> 32));
+                rec = decode_key(key, c, fd.w, fd.h, fd.gw, cv.h->levels, cv.h->cell_magic[0], cv.h->status);
                 *kp = 0;
                 hit = true;
-                const uint32_t magic = cv.h->cell_magic[0];
-                if (cv.h->status && (k >= cv.h->levels || rec.x >= fd.w || rec.y >= fd.h ||
-                                     __umulhi((uint32_t)rec.y, magic) * (uint32_t)fd.gw +
-                                             __umulhi((uint32_t)rec.x, magic) != (uint32_t)c))
-                    atomicOr(cv.h->status, kStatusBadKey);
             }
             sw->outs[s * nf + f][c] = rec;
             g = s * nf + f;

@@ -1,0 +1,209 @@
+// Host side of tile_detect_kernel: which calls it takes, their layout in the
+// resident buffers, and the launches.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cstring>
+
+#include "vio_ctx.h"
+#include "vio_tiles.cuh"
+
+using namespace vio;
+
+namespace {
+
+static_assert(kConsumers == 256, "block size of both kernels");
+
+// The kernels of a form for an NMS radius, by score.
+template <int CAP>
+struct TileKernel {
+    void (*fn[3])(TileCall<CAP>);
+    int tile_h, smem;
+};
+
+template <int SR, int R, int CAP>
+constexpr TileKernel<CAP> make_kernel() {
+    constexpr int TH = SR - 2 * R;
+    using G = TileGeom<TH, R>;
+    return {{tile_detect_kernel<TH, 0, R, CAP>, tile_detect_kernel<TH, 1, R, CAP>, tile_detect_kernel<TH, 2, R, CAP>},
+            TH,
+            G::BOXA + G::SR * G::SW * 2 + G::WARPS * G::QCAP * 2};
+}
+
+// Form 0: 32 score rows per tile, 4 per warp; form 1: 64 rows, 8 per warp.
+template <int FORM>
+const TileKernel<kTileCap[FORM]>& kernel_of(int radius) {
+    constexpr int SR = FORM == 0 ? 32 : 64, CAP = kTileCap[FORM];
+    static const TileKernel<CAP> k[4] = {make_kernel<SR, 1, CAP>(), make_kernel<SR, 2, CAP>(),
+                                         make_kernel<SR, 3, CAP>(), make_kernel<SR, 4, CAP>()};
+    return k[radius - 1];
+}
+
+// Which calls are taken, by their tiles (of the form in question); us per call,
+// the persistent three kernels against these launches:
+//   form 0, one launch     752x480, 3 levels, 280 tiles of 30 rows: 22.7 -> 10.6
+//                          1280x720: 20.4 -> 12.3; form 1 there 14.4 and 15.4
+//                          (but 8 frames 752x480, 1,200 tiles: form 1 17.0, form 0 20.6)
+//   form 1, one launch     16 mixed frames, 3 levels, 2,788 tiles: 60.4 -> 43.4 (two launches 50.0);
+//                          24, 4,182 tiles: 67.5 -> 59.4 (61.8); from 5,500 tiles on two are faster
+//   one level              16 mixed frames, 2,320 tiles: one launch 37.0, a decode launch of its own 34.8
+//   form 1, two launches   32 mixed frames, 5,576 tiles: 84.5 -> 77.3; 48, 8,364 tiles: 111.0 -> 110.2;
+//                          64, 11,152 tiles: 138.7 -> 141.3; 6 4K frames, 8,880 tiles: 72.8 -> 76.8
+//   unaligned frames       6 of 3001x2001, 6,694 tiles: 115.1 -> 103.9; 48 of 1021x765, 7,595: 125.0 -> 122.6
+// (a tile costs more here, 11 to 13 us per 1,000 of the mixed frames' against 9.4 in
+// the persistent kernel, whose loads run ahead; a call costs 7 to 20 us less to start).
+constexpr int kOneLaunch[2] = {800, 4000};  // forms 0 and 1, 2 or 3 levels of aligned frames
+constexpr int kOneLaunchOneLevel = 800;     // one level: form 1
+constexpr int kTwoLaunches[2] = {6000, 8000};  // aligned frames, others
+
+int tiles_of(const vio_dims& d, int k, int th) {
+    return (((d.w >> k) + kTileW - 1) / kTileW) * (((d.h >> k) + th - 1) / th);
+}
+
+template <int FORM>
+vio_status detect_form(vio_ctx* ctx, const uint8_t* const* lev0, const int* pitch0, const vio_dims* dims, int n,
+                       int thresh, int arc, int cell, int levels, int4* const* outs, int32_t* counts, cudaStream_t s,
+                       bool two) {
+    constexpr int CAP = kTileCap[FORM];
+    const TileKernel<CAP>& kern = kernel_of<FORM>(ctx->cfg.nms_radius);
+    const auto fn = kern.fn[ctx->cfg.score];
+    TileCall<CAP> c;
+    std::memset(&c, 0, offsetof(TileCall<CAP>, tiles));
+    size_t koff = 0, poff = 0;
+    for (int i = 0; i < n; ++i) {
+        FrameDesc& f = c.f[i];
+        std::memset(&f, 0, sizeof(f));
+        f.w = dims[i].w;
+        f.h = dims[i].h;
+        f.gw = (f.w + cell - 1) / cell;
+        f.gh = (f.h + cell - 1) / cell;
+        f.out = outs[i];
+        f.lev[0] = const_cast<uint8_t*>(lev0[i]);
+        f.pitch[0] = pitch0[i];
+        koff += align_up((size_t)f.gw * f.gh, 16);
+        for (int k = 1; k < levels; ++k) {
+            f.pitch[k] = (int)align_up(f.w >> k, 128);
+            poff += align_up((size_t)f.pitch[k] * (f.h >> k), 256);
+        }
+        for (int k = 0; k < levels; ++k) c.frame_tiles[i] += tiles_of(dims[i], k, kern.tile_h);
+    }
+    vio_status st;
+    const void* keys0 = ctx->d_keys;
+    const void* pyr0 = ctx->d_pyr;
+    if ((st = grow(ctx, (void**)&ctx->d_keys, &ctx->keys_cap, koff * 8, true)) != VIO_OK) return st;
+    if ((st = grow(ctx, (void**)&ctx->d_pyr, &ctx->pyr_cap, std::max<size_t>(poff, 256), false)) != VIO_OK) return st;
+    if (keys0 != ctx->d_keys || pyr0 != ctx->d_pyr) ctx->map_cache.clear();
+    koff = poff = 0;
+    for (int i = 0; i < n; ++i) {
+        FrameDesc& f = c.f[i];
+        f.keys = ctx->d_keys + koff;
+        koff += align_up((size_t)f.gw * f.gh, 16);
+        for (int k = 1; k < levels; ++k) {
+            f.lev[k] = ctx->d_pyr + poff;
+            poff += align_up((size_t)f.pitch[k] * (f.h >> k), 256);
+        }
+    }
+    c.thresh = thresh;
+    c.arc = arc;
+    c.n_frames = n;
+    c.levels = levels;
+    c.counts = counts;
+    c.done = two ? nullptr : ctx->d_done;
+    c.sums = ctx->d_sums;
+    c.status = ctx->d_status;
+    for (int k = 0; k < levels; ++k) {
+        const uint64_t d = (uint64_t)(cell >> k);
+        c.cell_magic[k] = (uint32_t)(((1ull << 32) + d - 1) / d);
+    }
+    // order against work of this context on another stream
+    if (ctx->have_last && ctx->last_stream != s) VIO_CK(cudaStreamWaitEvent(s, ctx->last_ev, 0));
+    if (!ctx->tile_ready[FORM]) {
+        VIO_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kern.smem));
+        ctx->tile_ready[FORM] = true;
+    }
+    const auto launch_grid = [&](void (*k)(TileCall<CAP>), int grid, int smem, bool dependent) -> vio_status {
+        cudaLaunchAttribute pdl[1];
+        pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        pdl[0].val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t lc = {};
+        lc.gridDim = dim3(grid);
+        lc.blockDim = dim3(256);
+        lc.dynamicSmemBytes = smem;
+        lc.stream = s;
+        lc.attrs = pdl;
+        lc.numAttrs = dependent ? 1 : 0;
+        VIO_CK(cudaLaunchKernelEx(&lc, k, c));
+        return VIO_OK;
+    };
+    const auto launch_levels = [&](int top, int n_levels, bool dependent) -> vio_status {
+        c.top = top;
+        c.n_levels = n_levels;
+        int acc = 0;
+        c.tiles[0] = 0;
+        for (int j = 0; j < n_levels; ++j)
+            for (int i = 0; i < n; ++i) c.tiles[j * n + i + 1] = acc += tiles_of(dims[i], top - j, kern.tile_h);
+        return launch_grid(fn, acc, kern.smem, dependent);
+    };
+    if (!two) {
+        if ((st = launch_levels(levels - 1, levels, false)) != VIO_OK) return st;
+    } else {
+        c.emit = std::min(levels - 1, 2);
+        if ((st = launch_levels(0, 1, false)) != VIO_OK) return st;
+        if (levels > 1) {
+            c.resident = c.emit;
+            c.emit = 0;
+            if ((st = launch_levels(levels - 1, levels - 1, true)) != VIO_OK) return st;
+        }
+        for (int i = 0; i < n; ++i) c.tiles[i + 1] = c.tiles[i] + (c.f[i].gw * c.f[i].gh + 255) / 256;
+        if ((st = launch_grid(tile_decode_kernel<CAP>, c.tiles[n], 0, true)) != VIO_OK) return st;
+    }
+    VIO_CK(cudaEventRecord(ctx->last_ev, s));
+    ctx->last_stream = s;
+    ctx->have_last = true;
+    ctx->last_levels = levels;
+    ctx->last_dims.assign(dims, dims + n);
+    ctx->last_lev.resize(n);
+    ctx->last_pitch.resize(n);
+    for (int i = 0; i < n; ++i)
+        for (int k = 0; k < levels; ++k) {
+            ctx->last_lev[i][k] = c.f[i].lev[k];
+            ctx->last_pitch[i][k] = c.f[i].pitch[k];
+        }
+    ctx->last_variant = ctx->default_variant;
+    ctx->last_ctas = 1;
+    ctx->last_cell = cell;
+    return VIO_OK;
+}
+
+}  // namespace
+
+namespace vio {
+
+vio_status detect_tiles(vio_ctx* ctx, const uint8_t* const* lev0, const int* pitch0, const vio_dims* dims, int n,
+                        int thresh, int arc, int cell, int levels, int4* const* outs, int32_t* counts, cudaStream_t s,
+                        bool* done) {
+    *done = false;
+    // a pinned or tuned launch shape and stage times ask for the three kernels
+    if (n > kTileCap[1] || ctx->cfg.profile || ctx->cfg.autotune || ctx->pinned_variant >= 0) return VIO_OK;
+    int tiles[2] = {0, 0};
+    const int th[2] = {kernel_of<0>(ctx->cfg.nms_radius).tile_h, kernel_of<1>(ctx->cfg.nms_radius).tile_h};
+    bool aligned = true;
+    for (int i = 0; i < n; ++i) {
+        aligned &= (((uintptr_t)lev0[i] | (uintptr_t)pitch0[i]) & 15) == 0;
+        for (int k = 0; k < levels; ++k)
+            for (int f = 0; f < 2; ++f) tiles[f] += tiles_of(dims[i], k, th[f]);
+    }
+    const bool one = levels <= 3 && aligned;
+    if (one && n <= kTileCap[0] && tiles[0] <= kOneLaunch[0]) {
+        *done = true;
+        return detect_form<0>(ctx, lev0, pitch0, dims, n, thresh, arc, cell, levels, outs, counts, s, false);
+    }
+    if (tiles[1] <= kTwoLaunches[aligned ? 0 : 1]) {
+        *done = true;
+        const bool two = !one || tiles[1] > (levels == 1 ? kOneLaunchOneLevel : kOneLaunch[1]);
+        return detect_form<1>(ctx, lev0, pitch0, dims, n, thresh, arc, cell, levels, outs, counts, s, two);
+    }
+    return VIO_OK;
+}
+
+}  // namespace vio
