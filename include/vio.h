@@ -448,8 +448,8 @@ typedef struct {
 void vio_track_params_default(vio_track_params* p);
 
 /*
- * Tracks n_pts[i] features from prev[i] to next[i] for i < n_pairs, one
- * launch for all pairs.
+ * Tracks n_pts[i] features from prev[i] to next[i] for i < n_pairs, one launch
+ * per 64 pairs.
  *
  *   prev, next  host arrays of n_pairs DEVICE pointers to uint8 frames; pair
  *               i has both frames of size dims[i] (pitch dims[i].pitch).

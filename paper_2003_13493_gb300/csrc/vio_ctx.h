@@ -73,11 +73,6 @@ constexpr int kHostSlots = 3;
 
 // Resident state of the feature tracker (vio_track).
 struct TrackState {
-    uint8_t* d_call = nullptr;   // the current call block
-    size_t call_cap = 0;
-    uint8_t* h_stage = nullptr;  // pinned staging of the call block
-    size_t stage_cap = 0;
-    cudaEvent_t stage_ev = nullptr;
     uint8_t* d_pyr = nullptr;    // levels 1..L-1 of both frames of every pair
     size_t pyr_cap = 0;
     uint8_t* d_in = nullptr;     // level-0 copies of frames that are not 16-byte aligned

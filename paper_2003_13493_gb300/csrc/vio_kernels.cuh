@@ -189,9 +189,52 @@ struct PyrRow {
     }
 };
 
+// Block `block` of a frame: 256 chunks, one per thread.
+template <int L>
+__device__ __forceinline__ void pyramid_block(const FrameDesc& fd, int block) {
+    constexpr int B = pyr_rows(L);
+    const int cx = fd.pyr_cx;
+    // chunk number = ty * cx + tx.  The product with ceil(2^32 / cx) gives
+    // the row of the block's first chunk or one more (at most 2^24 chunks
+    // of at most 2^12 per row), and exactly the row of a number below 2^13.
+    const int first = block * 256;
+    int row = (int)__umulhi((uint32_t)first, fd.pyr_magic);
+    if (row * cx > first) --row;
+    const int off = first - row * cx + (int)threadIdx.x;
+    const int down = (int)__umulhi((uint32_t)off, fd.pyr_magic);
+    const int tx = off - down * cx, ty = row + down;
+    const int W = fd.w, H = fd.h, x0 = tx * 16, y0 = ty * B;
+    if (x0 >= W || y0 >= H) return;
+    const bool upload = fd.src0 != nullptr;
+    const uint8_t* src = upload ? fd.src0 : fd.lev[0];
+    const int sp = upload ? fd.src0_pitch : fd.pitch[0];
+    const uint8_t* p = src + (size_t)y0 * sp + x0;
+    uint4 r[B];
+    if (x0 + 16 <= W && ((reinterpret_cast<uintptr_t>(src) | (uint32_t)sp) & 15) == 0) {
+#pragma unroll
+        for (int j = 0; j < B; ++j)
+            r[j] = y0 + j < H ? *reinterpret_cast<const uint4*>(p + (size_t)j * sp) : make_uint4(0, 0, 0, 0);
+    } else {
+        // the last partial chunk of a row, and frames of any alignment
+        const uint8_t* end = src + (size_t)sp * (H - 1) + W;
+#pragma unroll
+        for (int j = 0; j < B; ++j)
+            r[j] = y0 + j < H ? chunk_within(p + (size_t)j * sp, src, end) : make_uint4(0, 0, 0, 0);
+    }
+    if (upload) {
+#pragma unroll
+        for (int j = 0; j < B; ++j)
+            if (y0 + j < H) *reinterpret_cast<uint4*>(fd.lev[0] + (size_t)(y0 + j) * fd.pitch[0] + x0) = r[j];
+    }
+    if constexpr (L > 1) {
+        constexpr int TOP = L - 1;
+        PyrRow<TOP, B> top(fd, r, tx, ty, 0);
+        (void)top;
+    }
+}
+
 template <int L>
 __global__ void __launch_bounds__(256) pyramid_kernel(const uint8_t* __restrict__ call) {
-    constexpr int B = pyr_rows(L);
     griddep_launch_dependents();
     const CallView cv(call);
     const int nf = cv.h->n_frames, nb = cv.h->n_pyr_blocks;
@@ -205,45 +248,7 @@ __global__ void __launch_bounds__(256) pyramid_kernel(const uint8_t* __restrict_
     __syncthreads();
     for (int b = blockIdx.x; b < nb; b += gridDim.x) {
         const int f = upper_index(blocks, nf, b);
-        const FrameDesc& fd = cv.fds[f];
-        const int cx = fd.pyr_cx;
-        // chunk number = ty * cx + tx.  The product with ceil(2^32 / cx) gives
-        // the row of the block's first chunk or one more (at most 2^24 chunks
-        // of at most 2^12 per row), and exactly the row of a number below 2^13.
-        const int first = (b - blocks[f]) * 256;
-        int row = (int)__umulhi((uint32_t)first, fd.pyr_magic);
-        if (row * cx > first) --row;
-        const int off = first - row * cx + (int)threadIdx.x;
-        const int down = (int)__umulhi((uint32_t)off, fd.pyr_magic);
-        const int tx = off - down * cx, ty = row + down;
-        const int W = fd.w, H = fd.h, x0 = tx * 16, y0 = ty * B;
-        if (x0 >= W || y0 >= H) continue;
-        const bool upload = fd.src0 != nullptr;
-        const uint8_t* src = upload ? fd.src0 : fd.lev[0];
-        const int sp = upload ? fd.src0_pitch : fd.pitch[0];
-        const uint8_t* p = src + (size_t)y0 * sp + x0;
-        uint4 r[B];
-        if (x0 + 16 <= W && ((reinterpret_cast<uintptr_t>(src) | (uint32_t)sp) & 15) == 0) {
-#pragma unroll
-            for (int j = 0; j < B; ++j)
-                r[j] = y0 + j < H ? *reinterpret_cast<const uint4*>(p + (size_t)j * sp) : make_uint4(0, 0, 0, 0);
-        } else {
-            // the last partial chunk of a row, and frames of any alignment
-            const uint8_t* end = src + (size_t)sp * (H - 1) + W;
-#pragma unroll
-            for (int j = 0; j < B; ++j)
-                r[j] = y0 + j < H ? chunk_within(p + (size_t)j * sp, src, end) : make_uint4(0, 0, 0, 0);
-        }
-        if (upload) {
-#pragma unroll
-            for (int j = 0; j < B; ++j)
-                if (y0 + j < H) *reinterpret_cast<uint4*>(fd.lev[0] + (size_t)(y0 + j) * fd.pitch[0] + x0) = r[j];
-        }
-        if constexpr (L > 1) {
-            constexpr int TOP = L - 1;
-            PyrRow<TOP, B> top(fd, r, tx, ty, 0);
-            (void)top;
-        }
+        pyramid_block<L>(cv.fds[f], b - blocks[f]);
     }
 }
 

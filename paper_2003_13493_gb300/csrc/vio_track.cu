@@ -1,8 +1,9 @@
 // Host side of the feature tracker behind vio_track (Section II-E): argument
 // checks, the resident pyramid of both frames of every pair (built by the
-// detector's pyramid kernel), the per-call block and the launches.
+// detector's pyramid code) and the launches.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -15,16 +16,15 @@ using namespace vio;
 
 namespace {
 
-using PyrFn = void (*)(const uint8_t*);
-
-PyrFn track_pyr_fn(int levels) {
+// Launches of up to PAIRS pairs.
+template <int PAIRS>
+void (*track_pyr_fn(int levels))(TrackCall<PAIRS>) {
     switch (levels) {
-        case 1: return pyramid_kernel<1>;
-        case 2: return pyramid_kernel<2>;
-        case 3: return pyramid_kernel<3>;
-        case 4: return pyramid_kernel<4>;
-        case 5: return pyramid_kernel<5>;
-        default: return nullptr;
+        case 1: return track_pyramid_kernel<1, PAIRS>;
+        case 2: return track_pyramid_kernel<2, PAIRS>;
+        case 3: return track_pyramid_kernel<3, PAIRS>;
+        case 4: return track_pyramid_kernel<4, PAIRS>;
+        default: return track_pyramid_kernel<5, PAIRS>;
     }
 }
 
@@ -34,38 +34,103 @@ bool valid_params(const vio_track_params& p) {
            std::isfinite(p.min_update) && p.min_update >= 0.f && p.model >= 0 && p.model <= 3;
 }
 
-// Grows a pinned host buffer; the previous contents are not kept.
-vio_status grow_pinned(vio_ctx* ctx, uint8_t** p, size_t* cap, size_t need) {
-    if (need <= *cap && *p) return VIO_OK;
-    if (*p) {
-        VIO_CK(cudaFreeHost(*p));
-        *p = nullptr;
-        *cap = 0;
-    }
-    const size_t want = std::max(need, (size_t)4096);
-    VIO_CK(cudaHostAlloc((void**)p, want, cudaHostAllocDefault));
-    *cap = want;
-    return VIO_OK;
-}
-
 }  // namespace
 
 namespace vio {
 
 void track_release(vio_ctx* ctx) {
     TrackState& t = ctx->track;
-    if (t.stage_ev) cudaEventSynchronize(t.stage_ev);
-    if (t.d_call) cudaFree(t.d_call);
     if (t.d_pyr) cudaFree(t.d_pyr);
     if (t.d_in) cudaFree(t.d_in);
-    if (t.h_stage) cudaFreeHost(t.h_stage);
-    if (t.stage_ev) cudaEventDestroy(t.stage_ev);
     if (t.done_ev) cudaEventDestroy(t.done_ev);
-    ctx->bytes_in_use -= t.call_cap + t.pyr_cap + t.in_cap;
+    ctx->bytes_in_use -= t.pyr_cap + t.in_cap;
     t = TrackState{};
 }
 
 }  // namespace vio
+
+namespace {
+
+// Frame f of a call (2i: pair i's previous frame, 2i + 1 its next) and its place
+// in the resident buffers.
+struct TrackFrame {
+    const uint8_t* src;
+    size_t in_off;                 // (size_t)-1: read in place
+    size_t lev_off[kMaxLevels];
+};
+
+// Pairs [first, first + n) in one launch.
+template <int PAIRS>
+vio_status track_launch(vio_ctx* ctx, const vio_track_params& p, const TrackFrame* frames, const vio_dims* dims,
+                        int first, int n, const void* const* pts, const int* n_pts, vio_track_result* const* out,
+                        bool cells_in, cudaStream_t s) {
+    TrackState& T = ctx->track;
+    const int L = p.levels;
+    TrackCall<PAIRS> c;
+    c.levels = L;
+    c.patch_fine = p.patch_fine;
+    c.patch_coarse = p.patch_coarse;
+    c.max_iters = p.max_iters;
+    c.min_update = p.min_update;
+    c.model = p.model;
+    c.n_pairs = n;
+    c.cells_in = cells_in ? 1 : 0;
+    c.blocks[0] = 0;
+    c.prefix[0] = 0;
+    for (int i = 0; i < n; ++i) {
+        const vio_dims& d = dims[first + i];
+        c.pairs[i].pts = reinterpret_cast<const float*>(pts[first + i]);
+        c.pairs[i].out = reinterpret_cast<float*>(out[first + i]);
+        c.prefix[i + 1] = c.prefix[i] + n_pts[first + i];
+        for (int e = 0; e < 2; ++e) {
+            const TrackFrame& tf = frames[2 * (first + i) + e];
+            FrameDesc& fd = c.f[2 * i + e];
+            std::memset(&fd, 0, sizeof(fd));
+            fd.w = d.w;
+            fd.h = d.h;
+            if (tf.in_off != (size_t)-1) {
+                // copied by the pyramid kernel as it reads it
+                fd.src0 = tf.src;
+                fd.src0_pitch = d.pitch;
+                fd.lev[0] = T.d_in + tf.in_off;
+                fd.pitch[0] = (int)align_up(d.w, 16);
+            } else {
+                fd.lev[0] = const_cast<uint8_t*>(tf.src);
+                fd.pitch[0] = d.pitch;
+            }
+            for (int k = 1; k < L; ++k) {
+                fd.lev[k] = T.d_pyr + tf.lev_off[k];
+                fd.pitch[k] = (int)align_up(d.w >> k, 128);
+            }
+            c.blocks[2 * i + e + 1] = c.blocks[2 * i + e] + pyr_plan(fd, L);
+        }
+    }
+    c.n_features = c.prefix[n];
+    c.n_pyr_blocks = c.blocks[2 * n];
+    if (c.n_features == 0) return VIO_OK;
+    if (c.n_pyr_blocks > 0) {
+        // the kernel strides over its grid
+        const int grid = std::min(c.n_pyr_blocks, ctx->sm_count * 8);
+        track_pyr_fn<PAIRS>(L)<<<grid, 256, 0, s>>>(c);
+        VIO_CK(cudaGetLastError());
+    }
+    // few features are spread over the SMs, a warp or two each: a CTA's warps
+    // share an SM's pipes and its L1
+    const int warps = std::min(kTrackWarps, std::max(1, (c.n_features + ctx->sm_count - 1) / ctx->sm_count));
+    cudaLaunchAttribute pdl[1];
+    pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    pdl[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3((c.n_features + warps - 1) / warps);
+    lc.blockDim = dim3(warps * 32);
+    lc.stream = s;
+    lc.attrs = pdl;
+    lc.numAttrs = c.n_pyr_blocks > 0 ? 1 : 0;
+    VIO_CK(cudaLaunchKernelEx(&lc, track_kernel<PAIRS>, c));
+    return VIO_OK;
+}
+
+}  // namespace
 
 extern "C" {
 
@@ -83,9 +148,8 @@ void vio_track_params_default(vio_track_params* p) {
 namespace {
 
 vio_status track_impl(vio_ctx* ctx, const uint8_t* const* prev, const uint8_t* const* next, const vio_dims* dims,
-                      int n_pairs, const void* const* pts_in, const int* n_pts, const vio_track_params* params,
+                      int n_pairs, const void* const* pts, const int* n_pts, const vio_track_params* params,
                       vio_track_result* const* out, vio_stream stream, bool cells_in) {
-    const float* const* pts = reinterpret_cast<const float* const*>(pts_in);
     if (!ctx) return VIO_ERR_INVALID_ARG;
     vio_track_params p;
     if (params) p = *params; else vio_track_params_default(&p);
@@ -112,116 +176,39 @@ vio_status track_impl(vio_ctx* ctx, const uint8_t* const* prev, const uint8_t* c
     VIO_CK(cudaSetDevice(ctx->cfg.device));
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     TrackState& T = ctx->track;
-    const int nf = 2 * n_pairs;
 
     // resident layout: staged level-0 copies and levels 1..L-1 of every frame
-    std::vector<size_t> in_off(nf, (size_t)-1), lev_off(nf * kMaxLevels, 0);
-    std::vector<int> lev_pitch(nf * kMaxLevels, 0);
+    std::vector<TrackFrame> frames(2 * n_pairs);
     size_t ioff = 0, poff = 0;
-    for (int f = 0; f < nf; ++f) {
+    for (int f = 0; f < 2 * n_pairs; ++f) {
         const vio_dims& d = dims[f >> 1];
-        const uint8_t* src = (f & 1) ? next[f >> 1] : prev[f >> 1];
-        if (((uintptr_t)src & 15) || (d.pitch & 15)) {
-            in_off[f] = ioff;
+        TrackFrame& tf = frames[f];
+        tf.src = (f & 1) ? next[f >> 1] : prev[f >> 1];
+        tf.in_off = (size_t)-1;
+        if (((uintptr_t)tf.src & 15) || (d.pitch & 15)) {
+            tf.in_off = ioff;
             ioff += align_up(align_up(d.w, 16) * (size_t)d.h, 256);
         }
         for (int k = 1; k < L; ++k) {
-            lev_pitch[f * kMaxLevels + k] = (int)align_up(d.w >> k, 128);
-            lev_off[f * kMaxLevels + k] = poff;
-            poff += align_up((size_t)lev_pitch[f * kMaxLevels + k] * (d.h >> k), 256);
+            tf.lev_off[k] = poff;
+            poff += align_up(align_up(d.w >> k, 128) * (size_t)(d.h >> k), 256);
         }
     }
-    // call block sections
-    size_t off = align_up(sizeof(CallHeader), 128);
-    const size_t off_fds = off;
-    off += align_up(sizeof(FrameDesc) * nf, 128);
-    const size_t off_blocks = off;
-    off += align_up(sizeof(int32_t) * (nf + 1), 128);
-    const size_t off_track = off;
-    off += align_up(sizeof(TrackHeader), 128);
-    const size_t off_pairs = off;
-    off += align_up(sizeof(TrackPair) * n_pairs, 128);
-    const size_t off_prefix = off;
-    off += align_up(sizeof(int32_t) * (n_pairs + 1), 128);
-    const size_t bytes = off;
-
     vio_status st;
-    if (!T.stage_ev) VIO_CK(cudaEventCreateWithFlags(&T.stage_ev, cudaEventDisableTiming));
     if (!T.done_ev) VIO_CK(cudaEventCreateWithFlags(&T.done_ev, cudaEventDisableTiming));
-    VIO_CK(cudaEventSynchronize(T.stage_ev));  // the previous call's upload has left the staging buffer
     // the previous call's kernels read the device buffers this call rewrites
     if (T.have_done) VIO_CK(cudaStreamWaitEvent(s, T.done_ev, 0));
     if ((st = grow(ctx, (void**)&T.d_in, &T.in_cap, std::max<size_t>(ioff, 256), false)) != VIO_OK) return st;
     if ((st = grow(ctx, (void**)&T.d_pyr, &T.pyr_cap, std::max<size_t>(poff, 256), false)) != VIO_OK) return st;
-    if ((st = grow(ctx, (void**)&T.d_call, &T.call_cap, bytes, false)) != VIO_OK) return st;
-    if ((st = grow_pinned(ctx, &T.h_stage, &T.stage_cap, bytes)) != VIO_OK) return st;
-
-    uint8_t* hb = T.h_stage;
-    std::memset(hb, 0, bytes);
-    CallHeader* hdr = reinterpret_cast<CallHeader*>(hb);
-    FrameDesc* fds = reinterpret_cast<FrameDesc*>(hb + off_fds);
-    int32_t* blocks = reinterpret_cast<int32_t*>(hb + off_blocks);
-    TrackHeader* th = reinterpret_cast<TrackHeader*>(hb + off_track);
-    TrackPair* tps = reinterpret_cast<TrackPair*>(hb + off_pairs);
-    int32_t* prefix = reinterpret_cast<int32_t*>(hb + off_prefix);
-    hdr->n_frames = nf;
-    hdr->levels = L;
-    // the pyramid kernel reads only the frame descriptors and block prefix;
-    // the detector's other sections are empty here
-    hdr->off_fds = (uint32_t)off_fds;
-    hdr->off_blocks = (uint32_t)off_blocks;
-    hdr->off_maps0 = hdr->off_mapsk = hdr->off_tiles = hdr->off_cells = (uint32_t)off_blocks;
-    blocks[0] = 0;
-    for (int f = 0; f < nf; ++f) {
-        const vio_dims& d = dims[f >> 1];
-        const uint8_t* src = (f & 1) ? next[f >> 1] : prev[f >> 1];
-        FrameDesc& fd = fds[f];
-        fd.w = d.w;
-        fd.h = d.h;
-        if (in_off[f] != (size_t)-1) {
-            // copied by the pyramid kernel as it reads it
-            fd.src0 = src;
-            fd.src0_pitch = d.pitch;
-            fd.lev[0] = T.d_in + in_off[f];
-            fd.pitch[0] = (int)align_up(d.w, 16);
-        } else {
-            fd.lev[0] = const_cast<uint8_t*>(src);
-            fd.pitch[0] = d.pitch;
-        }
-        blocks[f + 1] = blocks[f] + pyr_plan(fd, L);
-        for (int k = 1; k < L; ++k) {
-            fd.lev[k] = T.d_pyr + lev_off[f * kMaxLevels + k];
-            fd.pitch[k] = lev_pitch[f * kMaxLevels + k];
-        }
+    if (n_pairs <= 8) {
+        if ((st = track_launch<8>(ctx, p, frames.data(), dims, 0, n_pairs, pts, n_pts, out, cells_in, s)) != VIO_OK)
+            return st;
+    } else {
+        for (int first = 0; first < n_pairs; first += 64)
+            if ((st = track_launch<64>(ctx, p, frames.data(), dims, first, std::min(64, n_pairs - first), pts, n_pts,
+                                       out, cells_in, s)) != VIO_OK)
+                return st;
     }
-    hdr->n_pyr_blocks = blocks[nf];
-    th->levels = L;
-    th->patch_fine = p.patch_fine;
-    th->patch_coarse = p.patch_coarse;
-    th->max_iters = p.max_iters;
-    th->min_update = p.min_update;
-    th->model = p.model;
-    th->n_pairs = n_pairs;
-    th->n_features = (int)total;
-    th->off_pairs = (uint32_t)off_pairs;
-    th->off_prefix = (uint32_t)off_prefix;
-    th->cells_in = cells_in ? 1 : 0;
-    prefix[0] = 0;
-    for (int i = 0; i < n_pairs; ++i) {
-        tps[i].pts = pts[i];
-        tps[i].out = reinterpret_cast<float*>(out[i]);
-        prefix[i + 1] = prefix[i] + n_pts[i];
-    }
-
-    VIO_CK(cudaMemcpyAsync(T.d_call, hb, bytes, cudaMemcpyHostToDevice, s));
-    VIO_CK(cudaEventRecord(T.stage_ev, s));
-    // the kernel strides over its grid: a few frames' blocks need no more than one CTA per SM
-    const int pyr_grid = blocks[nf] <= 2 * ctx->sm_count ? ctx->sm_count : ctx->sm_count * 8;
-    if (blocks[nf] > 0) track_pyr_fn(L)<<<pyr_grid, 256, 0, s>>>(T.d_call);
-    VIO_CK(cudaGetLastError());
-    const int grid = (int)((total + kTrackWarps - 1) / kTrackWarps);
-    track_kernel<<<grid, kTrackWarps * 32, 0, s>>>(T.d_call, (uint32_t)off_track);
-    VIO_CK(cudaGetLastError());
     VIO_CK(cudaEventRecord(T.done_ev, s));
     T.have_done = true;
     return VIO_OK;
