@@ -407,7 +407,7 @@ vio_status launch(vio_ctx* ctx, int variant, const uint8_t* const* lev0, const i
                   int ctas = 0) {
     const Variant& v = variants()[variant];
     // arena layout
-    size_t koff = 0, poff = 0;
+    size_t koff = 0, poff = ctx->group_pyr0;
     std::vector<size_t> key_off(n);
     std::vector<std::array<size_t, kMaxLevels>> lev_off(n);
     std::vector<std::array<int, kMaxLevels>> lev_pitch(n);
@@ -510,15 +510,7 @@ vio_status launch(vio_ctx* ctx, int variant, const uint8_t* const* lev0, const i
                 return st;
         }
     }
-    ctx->last_levels = levels;
-    ctx->last_dims.assign(dims, dims + n);
-    ctx->last_lev.assign(n, {});
-    ctx->last_pitch.assign(n, {});
-    for (int i = 0; i < n; ++i)
-        for (int k = 0; k < levels; ++k) {
-            ctx->last_lev[i][k] = fds[i].lev[k];
-            ctx->last_pitch[i][k] = fds[i].pitch[k];
-        }
+    remember_levels(ctx, fds, dims, n, levels);
     // tiles: coarsest level first, entry (L-1-k)*n + f
     int acc = 0;
     for (int kk = 0; kk < levels; ++kk) {
@@ -720,10 +712,97 @@ vio_status plan_staging(vio_ctx* ctx, const uint8_t* const* frames, const vio_di
 
 }  // namespace
 
+namespace {
+
+// A synchronous host call of this many bytes and more is detected in groups of
+// frames of about a sixth of it, at least kGroupMin bytes: while a group's
+// kernels run, the next group's copy is under way, so the call takes the upload
+// and the last group's kernels instead of the upload and then all kernels (64
+// mixed frames, 58.6 MB, whose upload alone takes 288 us: 444 -> 349 us; in 3,
+// 4 and 8 groups 377, 370 and 354 us; with last groups that halve, 373 us: a
+// group takes some 20 us however small).
+constexpr size_t kGroupBytes = 4u << 20, kGroupMin = 2u << 20;
+
+vio_status detect_in_groups(vio_ctx* ctx, const UploadPlan& plan, const uint8_t* const* host_frames,
+                            const vio_dims* dims, int n, int thresh, int arc, int cell, int levels, int4* const* outs,
+                            int32_t* d_counts, cudaStream_t s) {
+    vio_status st;
+    size_t total = 0, pyr = 0;
+    std::vector<size_t> pyr_at(n + 1, 0);
+    for (int i = 0; i < n; ++i) {
+        total += (size_t)dims[i].w * dims[i].h;
+        for (int k = 1; k < levels; ++k)
+            pyr += align_up(align_up(dims[i].w >> k, 128) * (size_t)(dims[i].h >> k), 256);
+        pyr_at[i + 1] = pyr;
+    }
+    // room for all groups' levels, so that no group grows the buffer
+    const void* pyr0 = ctx->d_pyr;
+    if ((st = grow(ctx, (void**)&ctx->d_pyr, &ctx->pyr_cap, std::max<size_t>(pyr, 256), false)) != VIO_OK) return st;
+    if (pyr0 != ctx->d_pyr) ctx->map_cache.clear();
+    if (!ctx->copy_stream) VIO_CK(cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking));
+    for (auto& e : ctx->group_ev)
+        if (!e) VIO_CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    // the copies follow the stream's work so far (it may write the host frames)
+    // and the context's previous call (it may read the staging buffer)
+    VIO_CK(cudaEventRecord(ctx->group_ev[0], s));
+    VIO_CK(cudaStreamWaitEvent(ctx->copy_stream, ctx->group_ev[0], 0));
+    if (ctx->have_last) VIO_CK(cudaStreamWaitEvent(ctx->copy_stream, ctx->last_ev, 0));
+    std::vector<const uint8_t*> lev0(n);
+    const size_t want = std::max(kGroupMin, total / 6 + 1);
+    for (int i = 0; i < n; ++i) lev0[i] = ctx->d_in + plan.off[i];
+    struct Reset {
+        vio_ctx* c;
+        ~Reset() {
+            c->group_pyr0 = 0;
+            c->group_follows = false;
+        }
+    } reset{ctx};
+    int copy = 0, copy_first = 0;  // the plan's current copy and its first frame
+    for (int first = 0, g = 0; first < n; ++g) {
+        size_t bytes = 0;
+        int end = first;
+        while (end < n && (g == kMaxGroups - 1 || end == first || bytes + (size_t)dims[end].w * dims[end].h <= want)) {
+            bytes += (size_t)dims[end].w * dims[end].h;
+            ++end;
+        }
+        // the group's part of the plan: whole copies, and its frames of a span
+        for (int i = first; i < end;) {
+            const UploadPlan::Copy& cp = plan.copies[copy];
+            const int copy_end = copy_first + plan.span_len[copy_first], j = std::min(end, copy_end);
+            if (cp.w == 0) {
+                const vio_dims& d = dims[j - 1];
+                const size_t part = (size_t)(host_frames[j - 1] + (size_t)d.pitch * (d.h - 1) + d.w - host_frames[i]);
+                VIO_CK(cudaMemcpyAsync(ctx->d_in + plan.off[i], host_frames[i], part, cudaMemcpyHostToDevice,
+                                       ctx->copy_stream));
+            } else {
+                VIO_CK(cudaMemcpy2DAsync(ctx->d_in + cp.dst, cp.dpitch, cp.src, cp.spitch, cp.w, cp.h,
+                                         cudaMemcpyHostToDevice, ctx->copy_stream));
+            }
+            i = j;
+            if (j == copy_end) {
+                copy_first = copy_end;
+                ++copy;
+            }
+        }
+        VIO_CK(cudaEventRecord(ctx->group_ev[1 + g], ctx->copy_stream));
+        VIO_CK(cudaStreamWaitEvent(s, ctx->group_ev[1 + g], 0));
+        ctx->group_pyr0 = pyr_at[first];
+        ctx->group_follows = first > 0;
+        if ((st = detect_impl(ctx, lev0.data() + first, plan.pitch.data() + first, dims + first, end - first, thresh,
+                              arc, cell, levels, outs + first, d_counts ? d_counts + first : nullptr, s)) != VIO_OK)
+            return st;
+        first = end;
+    }
+    return VIO_OK;
+}
+
+}  // namespace
+
 namespace vio {
 
 vio_status detect_from_host(vio_ctx* ctx, const uint8_t* const* host_frames, const vio_dims* dims, int n, int thresh,
-                            int arc, int cell, int levels, int4* const* outs, int32_t* d_counts, cudaStream_t s) {
+                            int arc, int cell, int levels, int4* const* outs, int32_t* d_counts, cudaStream_t s,
+                            bool may_group) {
     // Frames alone in pinned host memory, when a call has at least
     // kZeroCopyMin of them, are read by the pyramid kernel through their
     // device mapping (it writes the device copy of level 0 as it goes): their
@@ -751,8 +830,11 @@ vio_status detect_from_host(vio_ctx* ctx, const uint8_t* const* host_frames, con
         i += len;
     }
     const bool any_up = n_mapped >= kZeroCopyMin;
-    if (!any_up) std::fill(skip.begin(), skip.end(), false);
     for (int i = 0; i < n; ++i) lev0[i] = ctx->d_in + plan.off[i];
+    if (!any_up && may_group && n > 1 && plan.bytes >= kGroupBytes && !ctx->cfg.autotune && !ctx->cfg.profile &&
+        ctx->pinned_variant < 0)
+        return detect_in_groups(ctx, plan, host_frames, dims, n, thresh, arc, cell, levels, outs, d_counts, s);
+    if (!any_up) std::fill(skip.begin(), skip.end(), false);
     if ((st = enqueue_upload(ctx, plan, ctx->d_in, s, &skip)) != VIO_OK) return st;
     Upload up;
     if (any_up) {
@@ -935,6 +1017,9 @@ vio_status vio_destroy(vio_ctx* ctx) {
     for (auto& e : ctx->stage_ev)
         if (e) cudaEventDestroy(e);
     if (ctx->capture_stream) cudaStreamDestroy(ctx->capture_stream);
+    if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
+    for (auto& e : ctx->group_ev)
+        if (e) cudaEventDestroy(e);
     delete ctx;
     return VIO_OK;
 }
@@ -1080,8 +1165,8 @@ vio_status vio_detect_host(vio_ctx* ctx, const uint8_t* const* host_frames, cons
         outs[i] = direct_out[i] ? out_mapped : ctx->d_cells + coff[i];
     }
     int32_t* d_counts = reinterpret_cast<int32_t*>(ctx->d_cells + ncell_total);
-    if ((st = vio::detect_from_host(ctx, host_frames, dims, n, thresh, arc, cell, levels, outs.data(), d_counts, s)) !=
-        VIO_OK)
+    if ((st = vio::detect_from_host(ctx, host_frames, dims, n, thresh, arc, cell, levels, outs.data(), d_counts, s,
+                                    true)) != VIO_OK)
         return st;
     if (all_direct)
         VIO_CK(cudaMemcpyAsync(ctx->h_out + ncell_total * sizeof(int4), d_counts, sizeof(int32_t) * n,

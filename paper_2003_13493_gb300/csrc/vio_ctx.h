@@ -71,6 +71,8 @@ struct HostSlot {
 };
 constexpr int kHostSlots = 3;
 
+constexpr int kMaxGroups = 8;  // groups of a host call (vio_detect_host)
+
 // Resident state of the feature tracker (vio_track).
 struct TrackState {
     uint8_t* d_pyr = nullptr;    // levels 1..L-1 of both frames of every pair
@@ -154,6 +156,13 @@ struct vio_ctx {
     std::vector<std::array<int, vio::kMaxLevels>> last_pitch;
     std::vector<vio_dims> last_dims;
     int last_levels = 0;
+    // a call detected in groups of frames: where this group's pyramid begins in
+    // d_pyr, and whether it follows an earlier group, so that the levels of the
+    // whole call stay readable
+    size_t group_pyr0 = 0;
+    bool group_follows = false;
+    cudaStream_t copy_stream = nullptr;    // uploads of a grouped call
+    cudaEvent_t group_ev[1 + vio::kMaxGroups] = {};  // the call's start, then each group's upload
     vio::TrackState track;
     vio::HostSlot hslots[vio::kHostSlots];
     int hslot_pos = 0;
@@ -214,6 +223,28 @@ inline vio_status grow(vio_ctx* ctx, void** p, size_t* cap, size_t need, bool ze
 }  // namespace vio
 
 namespace vio {
+// Remembers the levels of a detection for vio_copy_level (after those of the
+// call's earlier groups).
+inline void remember_levels(vio_ctx* ctx, const FrameDesc* f, const vio_dims* dims, int n, int levels) {
+    if (!ctx->group_follows) {
+        ctx->last_dims.clear();
+        ctx->last_lev.clear();
+        ctx->last_pitch.clear();
+    }
+    ctx->last_levels = levels;
+    ctx->last_dims.insert(ctx->last_dims.end(), dims, dims + n);
+    for (int i = 0; i < n; ++i) {
+        std::array<const uint8_t*, kMaxLevels> lev{};
+        std::array<int, kMaxLevels> pitch{};
+        for (int k = 0; k < levels; ++k) {
+            lev[k] = f[i].lev[k];
+            pitch[k] = f[i].pitch[k];
+        }
+        ctx->last_lev.push_back(lev);
+        ctx->last_pitch.push_back(pitch);
+    }
+}
+
 // Frees the tracker's resident buffers (vio_destroy).
 void track_release(vio_ctx* ctx);
 }  // namespace vio
@@ -223,9 +254,12 @@ namespace vio {
 // are uploaded by the pyramid kernel through their device mapping, others by
 // the copy engines into the context's staging.  outs[i] may be device memory
 // or the device mapping of pinned host memory; d_counts is device memory or
-// nullptr.  Arguments are checked by the caller.
+// nullptr.  may_group: a large upload may be detected in groups of frames, the
+// copies of one beside the kernels of another.  Arguments are checked by the
+// caller.
 vio_status detect_from_host(vio_ctx* ctx, const uint8_t* const* host_frames, const vio_dims* dims, int n, int thresh,
-                            int arc, int cell, int levels, int4* const* outs, int32_t* d_counts, cudaStream_t s);
+                            int arc, int cell, int levels, int4* const* outs, int32_t* d_counts, cudaStream_t s,
+                            bool may_group = false);
 // Detects with tile_detect_kernel (vio_tiles.cuh) when the call is one that it
 // takes, and sets *done then.  Frames of any alignment, in device memory.
 vio_status detect_tiles(vio_ctx* ctx, const uint8_t* const* lev0, const int* pitch0, const vio_dims* dims, int n,

@@ -69,7 +69,7 @@ vio_status detect_form(vio_ctx* ctx, const uint8_t* const* lev0, const int* pitc
     const auto fn = kern.fn[ctx->cfg.score];
     TileCall<CAP> c;
     std::memset(&c, 0, offsetof(TileCall<CAP>, tiles));
-    size_t koff = 0, poff = 0;
+    size_t koff = 0, poff = ctx->group_pyr0;
     for (int i = 0; i < n; ++i) {
         FrameDesc& f = c.f[i];
         std::memset(&f, 0, sizeof(f));
@@ -93,7 +93,8 @@ vio_status detect_form(vio_ctx* ctx, const uint8_t* const* lev0, const int* pitc
     if ((st = grow(ctx, (void**)&ctx->d_keys, &ctx->keys_cap, koff * 8, true)) != VIO_OK) return st;
     if ((st = grow(ctx, (void**)&ctx->d_pyr, &ctx->pyr_cap, std::max<size_t>(poff, 256), false)) != VIO_OK) return st;
     if (keys0 != ctx->d_keys || pyr0 != ctx->d_pyr) ctx->map_cache.clear();
-    koff = poff = 0;
+    koff = 0;
+    poff = ctx->group_pyr0;
     for (int i = 0; i < n; ++i) {
         FrameDesc& f = c.f[i];
         f.keys = ctx->d_keys + koff;
@@ -160,15 +161,7 @@ vio_status detect_form(vio_ctx* ctx, const uint8_t* const* lev0, const int* pitc
     VIO_CK(cudaEventRecord(ctx->last_ev, s));
     ctx->last_stream = s;
     ctx->have_last = true;
-    ctx->last_levels = levels;
-    ctx->last_dims.assign(dims, dims + n);
-    ctx->last_lev.resize(n);
-    ctx->last_pitch.resize(n);
-    for (int i = 0; i < n; ++i)
-        for (int k = 0; k < levels; ++k) {
-            ctx->last_lev[i][k] = c.f[i].lev[k];
-            ctx->last_pitch[i][k] = c.f[i].pitch[k];
-        }
+    remember_levels(ctx, c.f, dims, n, levels);
     ctx->last_variant = ctx->default_variant;
     ctx->last_ctas = 1;
     ctx->last_cell = cell;
