@@ -44,17 +44,22 @@ const TileKernel<kTileCap[FORM]>& kernel_of(int radius) {
 //   form 0, one launch     752x480, 3 levels, 280 tiles of 30 rows: 22.7 -> 10.6
 //                          1280x720: 20.4 -> 12.3; form 1 there 14.4 and 15.4
 //                          (but 8 frames 752x480, 1,200 tiles: form 1 17.0, form 0 20.6)
-//   form 1, one launch     16 mixed frames, 3 levels, 2,788 tiles: 60.4 -> 43.4 (two launches 50.0);
-//                          24, 4,182 tiles: 67.5 -> 59.4 (61.8); from 5,500 tiles on two are faster
-//   one level              16 mixed frames, 2,320 tiles: one launch 37.0, a decode launch of its own 34.8
-//   form 1, two launches   32 mixed frames, 5,576 tiles: 84.5 -> 77.3; 48, 8,364 tiles: 111.0 -> 110.2;
-//                          64, 11,152 tiles: 138.7 -> 141.3; 6 4K frames, 8,880 tiles: 72.8 -> 76.8
-//   unaligned frames       6 of 3001x2001, 6,694 tiles: 115.1 -> 103.9; 48 of 1021x765, 7,595: 125.0 -> 122.6
+//   form 1, tiles of level 1 and 2 built from level 0
+//                          16 mixed frames, 3 levels, 2,788 tiles: 60.4 -> 39.3; 32, 5,576 tiles:
+//                          84.5 -> 72.5; 48, 8,364 tiles: 111.0 -> 109.1; 64, 11,152 tiles: 138.7 -> 143
+//   form 1, levels in two launches (more than 3 levels, or unaligned frames)
+//                          4 4K frames, 4 levels, 6,000 tiles: 63.6 -> 61.3; 6, 8,880 tiles: 72.8 -> 76.8;
+//                          6 of 3001x2001, 6,694 tiles: 115.1 -> 103.9; 48 of 1021x765, 7,595: 125.0 -> 122.6;
+//                          (16 and 48 mixed frames, 3 levels: 46.0 and 110.0)
 // (a tile costs more here, 11 to 13 us per 1,000 of the mixed frames' against 9.4 in
-// the persistent kernel, whose loads run ahead; a call costs 7 to 20 us less to start).
-constexpr int kOneLaunch[2] = {800, 4000};  // forms 0 and 1, 2 or 3 levels of aligned frames
-constexpr int kOneLaunchOneLevel = 800;     // one level: form 1
-constexpr int kTwoLaunches[2] = {6000, 8000};  // aligned frames, others
+// the persistent kernel, whose loads run ahead; a call costs up to 27 us less to start).
+constexpr int kFormTiles[2] = {800, 8000};      // aligned frames, at most 3 levels
+constexpr int kTwoStepTiles[2] = {6000, 8000};  // others: aligned, unaligned
+// A frame is decoded by the CTA of its last tile in a call of at most this many
+// tiles; above it a decode launch is faster than a fence and a count per tile
+// (8 1920x1080 frames, 3,040 tiles: 45.3 -> 42.5 us; 64 of 320x240, 1,088 tiles:
+// 22.7 either way).
+constexpr int kLastTileDecodes = 800;
 
 int tiles_of(const vio_dims& d, int k, int th) {
     return (((d.w >> k) + kTileW - 1) / kTileW) * (((d.h >> k) + th - 1) / th);
@@ -63,7 +68,7 @@ int tiles_of(const vio_dims& d, int k, int th) {
 template <int FORM>
 vio_status detect_form(vio_ctx* ctx, const uint8_t* const* lev0, const int* pitch0, const vio_dims* dims, int n,
                        int thresh, int arc, int cell, int levels, int4* const* outs, int32_t* counts, cudaStream_t s,
-                       bool two) {
+                       int tiles, bool two) {
     constexpr int CAP = kTileCap[FORM];
     const TileKernel<CAP>& kern = kernel_of<FORM>(ctx->cfg.nms_radius);
     const auto fn = kern.fn[ctx->cfg.score];
@@ -109,7 +114,8 @@ vio_status detect_form(vio_ctx* ctx, const uint8_t* const* lev0, const int* pitc
     c.n_frames = n;
     c.levels = levels;
     c.counts = counts;
-    c.done = two ? nullptr : ctx->d_done;
+    const bool decode_launch = two || tiles > kLastTileDecodes;
+    c.done = decode_launch ? nullptr : ctx->d_done;
     c.sums = ctx->d_sums;
     c.status = ctx->d_status;
     for (int k = 0; k < levels; ++k) {
@@ -155,6 +161,9 @@ vio_status detect_form(vio_ctx* ctx, const uint8_t* const* lev0, const int* pitc
             c.emit = 0;
             if ((st = launch_levels(levels - 1, levels - 1, true)) != VIO_OK) return st;
         }
+    }
+    if (decode_launch) {
+        c.tiles[0] = 0;
         for (int i = 0; i < n; ++i) c.tiles[i + 1] = c.tiles[i] + (c.f[i].gw * c.f[i].gh + 255) / 256;
         if ((st = launch_grid(tile_decode_kernel<CAP>, c.tiles[n], 0, true)) != VIO_OK) return st;
     }
@@ -187,14 +196,13 @@ vio_status detect_tiles(vio_ctx* ctx, const uint8_t* const* lev0, const int* pit
             for (int f = 0; f < 2; ++f) tiles[f] += tiles_of(dims[i], k, th[f]);
     }
     const bool one = levels <= 3 && aligned;
-    if (one && n <= kTileCap[0] && tiles[0] <= kOneLaunch[0]) {
+    if (one && n <= kTileCap[0] && tiles[0] <= kFormTiles[0]) {
         *done = true;
-        return detect_form<0>(ctx, lev0, pitch0, dims, n, thresh, arc, cell, levels, outs, counts, s, false);
+        return detect_form<0>(ctx, lev0, pitch0, dims, n, thresh, arc, cell, levels, outs, counts, s, tiles[0], false);
     }
-    if (tiles[1] <= kTwoLaunches[aligned ? 0 : 1]) {
+    if (tiles[1] <= (one ? kFormTiles[1] : kTwoStepTiles[aligned ? 0 : 1])) {
         *done = true;
-        const bool two = !one || tiles[1] > (levels == 1 ? kOneLaunchOneLevel : kOneLaunch[1]);
-        return detect_form<1>(ctx, lev0, pitch0, dims, n, thresh, arc, cell, levels, outs, counts, s, two);
+        return detect_form<1>(ctx, lev0, pitch0, dims, n, thresh, arc, cell, levels, outs, counts, s, tiles[1], !one);
     }
     return VIO_OK;
 }

@@ -125,15 +125,17 @@ __device__ __forceinline__ void emit_levels(const FrameDesc& fd, const ItemInfo&
 // The persistent kernel between a pyramid and a decode kernel costs a call about
 // 34 us whatever its size: the call block's upload, three launches, the ramp
 // and the tail of each.  Here
-//  - a call of up to some 4,000 tiles is one launch: a tile of level 1 or 2
+//  - with up to 3 levels all tiles are one launch: a tile of level 1 or 2
 //    builds its box from level 0 (with its halo, 1.35 times the level-0 bytes
-//    per level, from L2), so no tile waits for another and all run at once, and
-//    the CTA that finishes a frame's last tile decodes the frame;
-//  - a larger one is three: the tiles of level 0, which write levels 1 and 2 from
-//    their boxes; the others, which build levels 3 and 4 from level 2; the
-//    decode (each a programmatic dependent of the one before, so its CTAs move
-//    in as that drains; counting the finished tiles would cost each tile 0.9 us
-//    for its fence).
+//    per level, from L2), so no tile waits for another and all run at once;
+//  - with more (or frames that 16-byte loads cannot read) they are two: the tiles
+//    of level 0, which write levels 1 and 2 from their boxes, then the others,
+//    which build levels 3 and 4 from level 2;
+//  - the CTA that finishes a frame's last tile decodes the frame in the smallest
+//    calls, a decode launch in the others (counting the finished tiles costs each
+//    tile 0.9 us for its fence).
+// Each launch but the first is a programmatic dependent of the one before, so
+// its CTAs move in as that drains.
 // The phases of a tile are separated by CTA barriers, and the other four CTAs of
 // the SM fill them.  A tile alone takes 3.4 us (load 1.3, coarse test 0.6, full
 // test, scores and NMS 0.6, fence and count 0.9); the 280 tiles of a 752x480

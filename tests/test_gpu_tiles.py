@@ -57,6 +57,12 @@ def test_one_launch_builds_the_pyramid(n, levels):
           levels, pyramid=True)
 
 
+@pytest.mark.parametrize("levels", [1, 2, 3])
+def test_one_launch_and_a_decode_launch(levels):
+    """More than 800 tiles of 62 rows."""
+    check([(1920, 1080), (1921, 1083), (361, 129), (2000, 1100)], levels)
+
+
 @pytest.mark.parametrize("levels", [4, 5])
 @pytest.mark.parametrize("pad16", [True, False])
 def test_two_launches(levels, pad16):
