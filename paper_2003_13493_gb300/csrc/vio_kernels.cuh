@@ -146,9 +146,14 @@ __device__ __forceinline__ uint4 chunk_within(const uint8_t* p, const uint8_t* b
     const uint32_t a = (uint32_t)reinterpret_cast<uintptr_t>(p) & 3u, sh = 8u * a;
     const uint8_t* q = p - a;
     uint32_t w[5];
+    if (q >= begin && q + 20 <= end) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) w[i] = word_within(q + 4 * i, begin, end);
-    w[4] = a ? word_within(q + 16, begin, end) : 0u;
+        for (int i = 0; i < 5; ++i) w[i] = reinterpret_cast<const uint32_t*>(q)[i];
+    } else {  // at the ends of the frame
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[i] = word_within(q + 4 * i, begin, end);
+        w[4] = a ? word_within(q + 16, begin, end) : 0u;
+    }
     return make_uint4(__funnelshift_r(w[0], w[1], sh), __funnelshift_r(w[1], w[2], sh),
                       __funnelshift_r(w[2], w[3], sh), __funnelshift_r(w[3], w[4], sh));
 }
