@@ -166,8 +166,6 @@ ShapeKey shape_key(const vio_dims* dims, int n, int cell, int levels) {
     return k;
 }
 
-constexpr int kSmallDecodeCtas = 8;  // decode grid of a small call
-
 #define VIO_CK_STATUS(call)                \
     do {                                   \
         const vio_status s_ = (call);      \
@@ -189,13 +187,10 @@ vio_status fused_occupancy(vio_ctx* ctx, int variant, int* occ) {
 }
 
 // Enqueues pyramid -> fused detect -> decode on `s`; launch shapes depend only
-// on the context and on `small` (the kernels read the batch from the call
-// block and stride over whatever grid they get).  A small call (a few frames
-// of VGA size: at most one detect item, two pyramid blocks per SM) launches
-// one CTA per SM instead of filling every SM, which saves the start-up of CTAs
-// that would find no work.
+// on the context (the kernels read the batch from the call block and stride
+// over whatever grid they get).
 vio_status enqueue_kernels(vio_ctx* ctx, int variant, int levels, cudaStream_t s, bool pyramid = true,
-                           bool small = false, int ctas = 0) {
+                           int ctas = 0) {
     const Variant& v = variants()[variant];
     const int mode = ctx->cfg.score;
     const bool prof = ctx->cfg.profile != 0;
@@ -205,14 +200,14 @@ vio_status enqueue_kernels(vio_ctx* ctx, int variant, int levels, cudaStream_t s
     const unsigned rec_flags = cap == cudaStreamCaptureStatusActive ? cudaEventRecordExternal : 0u;
     if (prof) VIO_CK(cudaEventRecordWithFlags(ctx->stage_ev[0], s, rec_flags));
     if (pyramid) {
-        pyr_fn(levels)<<<ctx->sm_count * (small ? 1 : 8), 256, 0, s>>>(ctx->d_call);
+        pyr_fn(levels)<<<ctx->sm_count * 8, 256, 0, s>>>(ctx->d_call);
         VIO_CK(cudaGetLastError());
     }
     if (prof) VIO_CK(cudaEventRecordWithFlags(ctx->stage_ev[1], s, rec_flags));
     int occ = 0;
     VIO_CK_STATUS(fused_occupancy(ctx, variant, &occ));
     const int per_sm = ctas > 0 ? std::min(ctas, occ) : occ;
-    const int grid = small ? ctx->sm_count : per_sm * ctx->sm_count;
+    const int grid = per_sm * ctx->sm_count;
     // the detect kernel and the decode are programmatic dependents of the
     // kernel before them: they launch while it drains and wait for it on
     // the device (griddep_wait) before reading what it wrote
@@ -229,7 +224,7 @@ vio_status enqueue_kernels(vio_ctx* ctx, int variant, int levels, cudaStream_t s
     VIO_CK(cudaLaunchKernelEx(&lc, v.fn[mode], (const uint8_t*)ctx->d_call, ctx->d_counter, ctx->d_status));
     if (prof) VIO_CK(cudaEventRecordWithFlags(ctx->stage_ev[2], s, rec_flags));
     cudaLaunchConfig_t ld = lc;
-    ld.gridDim = dim3(small ? kSmallDecodeCtas : ctx->sm_count * 4);
+    ld.gridDim = dim3(ctx->sm_count * 4);
     ld.blockDim = dim3(256);
     ld.dynamicSmemBytes = 0;
     VIO_CK(cudaLaunchKernelEx(&ld, decode_kernel, (const uint8_t*)ctx->d_call, ctx->d_counter));
@@ -240,9 +235,9 @@ vio_status enqueue_kernels(vio_ctx* ctx, int variant, int levels, cudaStream_t s
 // Graph slot `levels` holds pyramid -> detect -> decode (with one level the
 // pyramid kernel only stages frames); slot 0 holds detect -> decode alone (the
 // pyramid is already in place, or there is nothing to build or stage).
-vio_status get_graph(vio_ctx* ctx, int variant, int levels, bool pyramid, bool small, int ctas,
+vio_status get_graph(vio_ctx* ctx, int variant, int levels, bool pyramid, int ctas,
                      cudaGraphExec_t* out) {
-    cudaGraphExec_t& g = ctx->graphs[variant][pyramid ? levels : 0][small ? 1 : 0][ctas];
+    cudaGraphExec_t& g = ctx->graphs[variant][pyramid ? levels : 0][ctas];
     if (!g) {
         // the launch attributes and the occupancy are set up outside the capture
         int occ = 0;
@@ -250,7 +245,7 @@ vio_status get_graph(vio_ctx* ctx, int variant, int levels, bool pyramid, bool s
         (void)occ;
         cudaGraph_t graph = nullptr;
         VIO_CK(cudaStreamBeginCapture(ctx->capture_stream, cudaStreamCaptureModeThreadLocal));
-        vio_status es = enqueue_kernels(ctx, variant, levels, ctx->capture_stream, pyramid, small, ctas);
+        vio_status es = enqueue_kernels(ctx, variant, levels, ctx->capture_stream, pyramid, ctas);
         cudaError_t ce = cudaStreamEndCapture(ctx->capture_stream, &graph);
         if (es != VIO_OK) return es;
         VIO_CK(ce);
@@ -540,9 +535,6 @@ vio_status launch(vio_ctx* ctx, int variant, const uint8_t* const* lev0, const i
         for (int j = 0; j < n_set * n; ++j) so[j] = sweep->outs[j];
     }
 
-    const bool small = acc <= ctx->sm_count && blocks[n] <= 2 * ctx->sm_count &&
-                       cells[n] <= kSmallDecodeCtas * 256 * 4;
-
     pyramid = pyramid && blocks[n] > 0;
     VIO_CK(cudaMemcpyAsync(ctx->d_call, st_base, bytes, cudaMemcpyHostToDevice, s));
     VIO_CK(cudaEventRecord(ctx->ring_ev[slot], s));
@@ -552,9 +544,9 @@ vio_status launch(vio_ctx* ctx, int variant, const uint8_t* const* lev0, const i
             return st;
     } else if (ctx->cfg.use_graphs) {
         cudaGraphExec_t g = nullptr;
-        if ((st = get_graph(ctx, variant, levels, pyramid, small, ctas, &g)) != VIO_OK) return st;
+        if ((st = get_graph(ctx, variant, levels, pyramid, ctas, &g)) != VIO_OK) return st;
         VIO_CK(cudaGraphLaunch(g, s));
-    } else if ((st = enqueue_kernels(ctx, variant, levels, s, pyramid, small, ctas)) != VIO_OK) {
+    } else if ((st = enqueue_kernels(ctx, variant, levels, s, pyramid, ctas)) != VIO_OK) {
         return st;
     }
     VIO_CK(cudaEventRecord(ctx->last_ev, s));
@@ -564,7 +556,7 @@ vio_status launch(vio_ctx* ctx, int variant, const uint8_t* const* lev0, const i
     if (!sweep) VIO_CK_STATUS(fused_occupancy(ctx, variant, &occ));
     // a sweep's launch shape is fixed: the CTAs per SM its registers and
     // shared memory allow
-    ctx->last_ctas = sweep ? ctx->grid_sweep / ctx->sm_count : small ? 1 : (ctas > 0 ? std::min(ctas, occ) : occ);
+    ctx->last_ctas = sweep ? ctx->grid_sweep / ctx->sm_count : (ctas > 0 ? std::min(ctas, occ) : occ);
     ctx->last_cell = cell;
     return VIO_OK;
 }

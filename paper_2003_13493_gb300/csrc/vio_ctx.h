@@ -131,10 +131,9 @@ struct vio_ctx {
     cudaStream_t last_stream = nullptr;
     bool have_last = false;
 
-    // one graph per (variant, levels, launch shape, CTAs per SM): every batch
-    // shape replays it; shape 1 is the small-call shape (one CTA per SM at
-    // most); CTAs per SM 0 = as many as fit
-    cudaGraphExec_t graphs[8][vio::kMaxLevels + 1][2][vio::kMaxCtasPerSm + 1] = {};
+    // one graph per (variant, levels, CTAs per SM): every batch shape replays
+    // it; CTAs per SM 0 = as many as fit
+    cudaGraphExec_t graphs[8][vio::kMaxLevels + 1][vio::kMaxCtasPerSm + 1] = {};
     int occ_fused[8] = {};                 // CTAs per SM that fit, per variant
     int grid_sweep = 0;
     bool tile_ready[2] = {};               // attributes of the two forms of tile_detect_kernel are set
@@ -169,13 +168,12 @@ struct vio_ctx {
 
     void drop_graphs() {
         for (auto& row : graphs)
-            for (auto& pair : row)
-                for (auto& shape : pair)
-                    for (auto& g : shape)
-                        if (g) {
-                            cudaGraphExecDestroy(g);
-                            g = nullptr;
-                        }
+            for (auto& shape : row)
+                for (auto& g : shape)
+                    if (g) {
+                        cudaGraphExecDestroy(g);
+                        g = nullptr;
+                    }
     }
 };
 
