@@ -36,16 +36,6 @@ constexpr int kTrackMaxGrid = 18 * 18;
 // that is a multiple of 8, three or four 8-byte loads per lane.
 constexpr int kWinRows = 25, kWinCols = 32, kWinUnits = kWinRows * kWinCols / 8, kWinLoads = (kWinUnits + 31) / 32;
 
-// Bilinear sample of an 8-bit image at (x, y), 0 <= x <= W-2, 0 <= y <= H-2.
-__device__ __forceinline__ float bilinear(const uint8_t* img, int pitch, float x, float y) {
-    const float fx = floorf(x), fy = floorf(y);
-    const float ax = x - fx, ay = y - fy;
-    const uint8_t* p = img + (size_t)(int)fy * pitch + (int)fx;
-    const float a = p[0], b = p[1], c = p[pitch], d = p[pitch + 1];
-    const float top = fmaf(ax, b - a, a), bot = fmaf(ax, d - c, c);
-    return fmaf(ay, bot - top, top);
-}
-
 __device__ __forceinline__ bool inside(float x, float y, int w, int h) {
     return x >= 0.f && y >= 0.f && x <= (float)(w - 2) && y <= (float)(h - 2);
 }
@@ -159,27 +149,35 @@ struct TrackLevel {
     int pitch_prev, pitch_next, w, h;
 };
 
-// The window's place around the pixels c0 - 1 .. c0 + need, r0 - 1 .. r0 + need
-// of a w x h image: as central as its alignment allows; ok false in an image
-// smaller than the window.  (The levels are written by the kernel before this
-// one, which may run when this one starts, so they are read by plain loads and
-// not as read-only data.)
+// A window's place in a w x h image, so that it holds the pixels c0 - 1 ..
+// c0 + need, r0 - 1 .. r0 + need that the image has: central, its column a
+// multiple of 8, but not beyond the image (an image smaller than the window
+// fills a part of it).  (The levels are written by the kernel before this one,
+// which may run when this one starts, so they are read by plain loads and not as
+// read-only data.)
 struct Window {
     int x, y, w, h;
-    bool ok;
     __device__ __forceinline__ static Window around(int c0, int r0, int need, int w, int h) {
         Window v;
-        v.x = max(0, min(c0 - max(1, (kWinCols - 8 - need) / 2), w - kWinCols)) & ~7;
-        v.y = max(0, min(r0 - max(1, (kWinRows - need) / 2), h - kWinRows));
+        v.x = max(0, c0 - max(1, (kWinCols - 8 - need) / 2)) & ~7;
+        if (v.x + kWinCols > w) {
+            // the last whole place, if that reaches far enough, or the border
+            v.x = max(0, w - kWinCols);
+            const int a = v.x & ~7;
+            if (min(c0 + need, w - 1) < a + kWinCols) v.x = a;
+        }
+        v.y = min(max(0, r0 - max(1, (kWinRows - need) / 2)), max(0, h - kWinRows));
         v.w = w;
         v.h = h;
-        v.ok = w >= kWinCols && h >= kWinRows;
         return v;
     }
-    // all of columns c0 - 1 .. c0 + need and rows r0 - 1 .. r0 + need that the image has
     __device__ __forceinline__ bool holds(int c0, int r0, int need) const {
-        return ok && max(0, c0 - 1) >= x && min(c0 + need, w - 1) < x + kWinCols && max(0, r0 - 1) >= y &&
+        return max(0, c0 - 1) >= x && min(c0 + need, w - 1) < x + kWinCols && max(0, r0 - 1) >= y &&
                min(r0 + need, h - 1) < y + kWinRows;
+    }
+    // 8-byte loads stay inside the rows and start where they must
+    __device__ __forceinline__ bool whole() const {
+        return (x & 7) == 0 && x + kWinCols <= w && y + kWinRows <= h;
     }
 };
 
@@ -189,7 +187,7 @@ __device__ __forceinline__ void window_load(const Window& v, const uint8_t* img,
     for (int i = 0; i < kWinLoads; ++i) {
         const int u = lane + 32 * i;
         w[i] = make_uint2(0, 0);
-        if (v.ok && u < kWinUnits)
+        if (u < kWinUnits)
             w[i] = *reinterpret_cast<const uint2*>(img + (size_t)(v.y + (u >> 2)) * pitch + v.x + 8 * (u & 3));
     }
 }
@@ -200,6 +198,21 @@ __device__ __forceinline__ void window_store(const uint2 (&w)[kWinLoads], uint8_
         const int u = lane + 32 * i;
         if (u < kWinUnits) *reinterpret_cast<uint2*>(win + 8 * u) = w[i];
     }
+}
+
+// A window at the right or lower border, or of a small image, byte by byte (a
+// lane per column); out of line, so that the loops stay short.
+__device__ __noinline__ void window_bytes(const Window& v, const uint8_t* img, int pitch, int lane, uint8_t* win) {
+    const int rows = min(kWinRows, v.h - v.y);
+    if (v.x + lane < v.w) {
+        const uint8_t* p = img + (size_t)v.y * pitch + v.x + lane;
+        uint8_t b[kWinRows];
+#pragma unroll
+        for (int r = 0; r < kWinRows; ++r) b[r] = r < rows ? p[(size_t)r * pitch] : (uint8_t)0;
+#pragma unroll
+        for (int r = 0; r < kWinRows; ++r) win[r * kWinCols + lane] = b[r];
+    }
+    __syncwarp();
 }
 
 // Per warp: the template grid and the windows of both images.
@@ -217,12 +230,14 @@ __device__ __forceinline__ float to_float(uint8_t v) { return __uint2float_rn((u
 // A feature is a chain of latencies: per level the template's pixels, the
 // factorisation, and per iteration the samples, the sums and the solve.  The
 // pixels of both images around the feature come to shared memory once per level
-// with all loads in flight at once (again when the track leaves the window; near
-// the border samples come from memory), the sums and the divisions share the
-// lanes.  (With byte loads from memory in every iteration, 25 shuffles for the
+// with all loads in flight at once (again when the track leaves the window), the
+// sums and the divisions share the lanes.  (With byte loads from memory in every iteration, 25 shuffles for the
 // five sums and a chain of ten divisions a 16 x 16 level took 4,800 cycles for
 // the template, 2,000 for the factor and 1,700 per iteration; 100 features
-// 30.9 -> 14.4 us a call, 64 pairs x 256 features 131 -> 108 us.)
+// 30.9 -> 14.0 us a call, 64 pairs x 256 features 131 -> 102 us.  Sampling from
+// memory where a window does not fit kept a second copy of every loop: a lone
+// warp then waits for its instructions, and the detect-then-track loop took 45.5
+// instead of 36.9 us a frame.)
 template <int P>
 __device__ bool track_level(const TrackLevel& lv, float cx, float cy, TrackShared& sh, int lane, int model,
                             int max_iters, float min_update, float& tx, float& ty, float& alpha, float& beta,
@@ -241,32 +256,29 @@ __device__ bool track_level(const TrackLevel& lv, float cx, float cy, TrackShare
     // (a position far outside the image overflows nothing: it is clamped, and no sample is taken)
     const auto cell = [](float v) { return (int)floorf(fminf(fmaxf(v, -1e6f), 1e6f)); };
     Window wn = Window::around(cell(o0 + tx), cell(o1 + ty), P + 2, lv.w, lv.h);
-    {
+    if (wp.whole() && wn.whole()) {
         uint2 a[kWinLoads], b[kWinLoads];
         window_load(wp, lv.prev, lv.pitch_prev, lane, a);
         window_load(wn, lv.next, lv.pitch_next, lane, b);
         window_store(a, sh.prev, lane);
         window_store(b, sh.next, lane);
+    } else {
+        window_bytes(wp, lv.prev, lv.pitch_prev, lane, sh.prev);
+        window_bytes(wn, lv.next, lv.pitch_next, lane, sh.next);
     }
     __syncwarp();
-    const bool staged = wp.holds(pc, pr, G + 1);
 #pragma unroll
     for (int k = 0; k < GS; ++k) {
         const int idx = lane + 32 * k;
         if (idx < G * G) {
             const int j = idx / G, i = idx - j * G;
             const float gx = o0 - 1.f + (float)i, gy = o1 - 1.f + (float)j;
-            if (staged) {
-                const float fx = floorf(gx), fy = floorf(gy);
-                const float ax = gx - fx, ay = gy - fy;
-                const uint8_t* p = sh.prev + ((int)fy - wp.y) * kWinCols + ((int)fx - wp.x);
-                const float a = to_float(p[0]), b = to_float(p[1]), c = to_float(p[kWinCols]),
-                            d = to_float(p[kWinCols + 1]);
-                const float top = fmaf(ax, b - a, a), bot = fmaf(ax, d - c, c);
-                sh.grid[idx] = fmaf(ay, bot - top, top);
-            } else {
-                sh.grid[idx] = bilinear(lv.prev, lv.pitch_prev, gx, gy);
-            }
+            const float fx = floorf(gx), fy = floorf(gy);
+            const float ax = gx - fx, ay = gy - fy;
+            const uint8_t* p = sh.prev + ((int)fy - wp.y) * kWinCols + ((int)fx - wp.x);
+            const float a = to_float(p[0]), b = to_float(p[1]), c = to_float(p[kWinCols]), d = to_float(p[kWinCols + 1]);
+            const float top = fmaf(ax, b - a, a), bot = fmaf(ax, d - c, c);
+            sh.grid[idx] = fmaf(ay, bot - top, top);
         }
     }
     __syncwarp();
@@ -328,40 +340,21 @@ __device__ bool track_level(const TrackLevel& lv, float cx, float cy, TrackShare
             return false;
         }
         const int c0 = (int)floorf(x_lo), r0 = (int)floorf(y_lo);
-        bool in_window = wn.holds(c0, r0, P + 2);
-        if (!in_window) {
-            // the track has left the window: move it, once per place
-            const Window moved = Window::around(c0, r0, P + 2, lv.w, lv.h);
-            if (moved.holds(c0, r0, P + 2)) {
-                wn = moved;
-                uint2 b[kWinLoads];
-                window_load(wn, lv.next, lv.pitch_next, lane, b);
-                __syncwarp();
-                window_store(b, sh.next, lane);
-                __syncwarp();
-                in_window = true;
-            }
+        if (!wn.holds(c0, r0, P + 2)) {  // the track has left the window
+            wn = Window::around(c0, r0, P + 2, lv.w, lv.h);
+            __syncwarp();
+            window_bytes(wn, lv.next, lv.pitch_next, lane, sh.next);
         }
         // this lane's samples: column xs, rows ys .. ys + NPX - 1 of the next image
         const float xs = o0 + (float)col + tx, ys = o1 + (float)row0 + ty;
         const float fx = floorf(xs), fy = floorf(ys);
         const float ax = xs - fx, ay = ys - fy;
+        const uint8_t* q = sh.next + ((int)fy - wn.y) * kWinCols + ((int)fx - wn.x);
         float p0[NPX + 1], p1[NPX + 1];
-        if (in_window) {
-            const uint8_t* q = sh.next + ((int)fy - wn.y) * kWinCols + ((int)fx - wn.x);
 #pragma unroll
-            for (int m = 0; m <= NPX; ++m) {
-                p0[m] = to_float(q[m * kWinCols]);
-                p1[m] = to_float(q[m * kWinCols + 1]);
-            }
-        } else {
-            const uint8_t* q = lv.next + (size_t)(int)fy * lv.pitch_next + (int)fx;
-#pragma unroll
-            for (int m = 0; m <= NPX; ++m) {
-                p0[m] = to_float(q[0]);
-                p1[m] = to_float(q[1]);
-                q += lv.pitch_next;
-            }
+        for (int m = 0; m <= NPX; ++m) {
+            p0[m] = to_float(q[m * kWinCols]);
+            p1[m] = to_float(q[m * kWinCols + 1]);
         }
         float top = fmaf(ax, p1[0] - p0[0], p0[0]);
         float b[5] = {0.f, 0.f, 0.f, 0.f, 0.f};  // U r, and the squared residual

@@ -78,3 +78,29 @@ def test_tracking_of_unaligned_pairs(levels):
     assert all(np.array_equal(g.view(np.int32), got[0].view(np.int32)) for g in got)
     assert (got[0].view(np.int32)[:, 4] == 1).mean() > 0.9
     det.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("size", [(40, 31), (23, 300), (300, 24), (33, 26), (96, 64)])
+def test_tracking_near_borders_and_in_small_images(size):
+    """Features everywhere, also where the pixel windows reach the border or the image is smaller than
+    one: status as the oracle's, positions of the tracked ones (fixed iterations)."""
+    torch = pytest.importorskip("torch")
+    from oracle import lk_oracle as lk
+    w, h = size
+    a, b = synth.smooth_frame(w, h, 8), synth.smooth_frame(w, h, 8, dx=0.75, dy=-0.5)
+    pts = np.array([[x, y] for y in np.arange(2.25, h - 2, 3.5) for x in np.arange(2.5, w - 2, 3.25)], np.float32)
+    det = vio.Detector(max_frames=2)
+    for levels in (1, 2) if min(w, h) >= 16 else (1,):
+        p = dict(patch_fine=8, patch_coarse=8, max_iters=6, min_update=0.0, model=0)
+        got = det.track([place(torch, a, 0, w + (-w) % 16)], [place(torch, b, 0, w + (-w) % 16)],
+                        [torch.from_numpy(pts).cuda()], dict(p, levels=levels))[0].cpu().numpy()
+        want = lk.track(a, b, pts.astype(np.float64), levels=levels, **p)
+        status = got.view(np.int32)[:, 4]
+        # a position that fp32 rounds across a border may flip a track near it
+        assert (status != want[:, 4].astype(np.int32)).mean() <= 0.01
+        more = lk.track(a, b, pts.astype(np.float64), levels=levels, **dict(p, max_iters=7))
+        ok = (status == 1) & (want[:, 4] == 1) & (np.abs(want[:, :2] - more[:, :2]).max(axis=1) < 1e-6)
+        # (on two levels every patch of the narrow images leaves the coarse one)
+        assert (ok.sum() > 0 or levels == 2) and np.abs(got[ok, :2] - want[ok, :2]).max(initial=0) < 1e-3
+    det.close()
