@@ -622,12 +622,10 @@ vio_status autotune(vio_ctx* ctx, const ShapeKey& key, const uint8_t* const* lev
 vio_status detect_impl(vio_ctx* ctx, const uint8_t* const* lev0, const int* pitch0, const vio_dims* dims, int n,
                        int thresh, int arc, int cell, int levels, int4* const* outs, int32_t* counts,
                        cudaStream_t s, Upload up = {}) {
-    if (!up.src) {
-        bool done = false;
-        const vio_status st = vio::detect_tiles(ctx, lev0, pitch0, dims, n, thresh, arc, cell ? cell : 32, levels, outs,
-                                                counts, s, &done);
-        if (st != VIO_OK || done) return st;
-    }
+    bool done = false;
+    const vio_status st_tiles = vio::detect_tiles(ctx, lev0, pitch0, dims, n, thresh, arc, cell ? cell : 32, levels,
+                                                  outs, counts, s, &done, up.src, up.pitch);
+    if (st_tiles != VIO_OK || done) return st_tiles;
     int vi = ctx->pinned_variant;
     int ctas = ctx->pinned_ctas;
     int c = cell ? cell : 32;

@@ -259,10 +259,12 @@ vio_status detect_from_host(vio_ctx* ctx, const uint8_t* const* host_frames, con
                             int arc, int cell, int levels, int4* const* outs, int32_t* d_counts, cudaStream_t s,
                             bool may_group = false);
 // Detects with tile_detect_kernel (vio_tiles.cuh) when the call is one that it
-// takes, and sets *done then.  Frames of any alignment, in device memory.
+// takes, and sets *done then.  Frames of any alignment, in device memory; with
+// src, frames whose src[i] is not nullptr (row pitch src_pitch[i]) are first
+// copied to lev0[i] by the pyramid kernel, as by vio_api.cu's Upload.
 vio_status detect_tiles(vio_ctx* ctx, const uint8_t* const* lev0, const int* pitch0, const vio_dims* dims, int n,
                         int thresh, int arc, int cell, int levels, int4* const* outs, int32_t* counts, cudaStream_t s,
-                        bool* done);
+                        bool* done, const uint8_t* const* src = nullptr, const int* src_pitch = nullptr);
 // Device address of pinned host memory, else nullptr.
 const void* host_device_alias(const void* host);
 }  // namespace vio

@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstddef>
 #include <cstring>
 
 #include "vio_ctx.h"
@@ -39,6 +40,17 @@ const TileKernel<kTileCap[FORM]>& kernel_of(int radius) {
     return k[radius - 1];
 }
 
+template <int CAP>
+void (*pyramid_of(int levels))(TileCall<CAP>) {
+    switch (levels) {
+        case 1: return tile_pyramid_kernel<1, CAP>;
+        case 2: return tile_pyramid_kernel<2, CAP>;
+        case 3: return tile_pyramid_kernel<3, CAP>;
+        case 4: return tile_pyramid_kernel<4, CAP>;
+        default: return tile_pyramid_kernel<5, CAP>;
+    }
+}
+
 // Which calls are taken, by their tiles (of the form in question); us per call,
 // the persistent three kernels against these launches:
 //   form 0, one launch     752x480, 3 levels, 280 tiles of 30 rows: 22.7 -> 10.6
@@ -51,6 +63,8 @@ const TileKernel<kTileCap[FORM]>& kernel_of(int radius) {
 //                          4 4K frames, 4 levels, 6,000 tiles: 63.6 -> 61.3; 6, 8,880 tiles: 72.8 -> 76.8;
 //                          6 of 3001x2001, 6,694 tiles: 115.1 -> 103.9; 48 of 1021x765, 7,595: 125.0 -> 122.6;
 //                          (16 and 48 mixed frames, 3 levels: 46.0 and 110.0)
+//   form 1 after a pyramid kernel that uploads the frames
+//                          16 pinned frames, host call: 140 -> 127; 8: 87.5 -> 82
 // (a tile costs more here, 11 to 13 us per 1,000 of the mixed frames' against 9.4 in
 // the persistent kernel, whose loads run ahead; a call costs up to 27 us less to start).
 constexpr int kFormTiles[2] = {800, 8000};      // aligned frames, at most 3 levels
@@ -68,12 +82,12 @@ int tiles_of(const vio_dims& d, int k, int th) {
 template <int FORM>
 vio_status detect_form(vio_ctx* ctx, const uint8_t* const* lev0, const int* pitch0, const vio_dims* dims, int n,
                        int thresh, int arc, int cell, int levels, int4* const* outs, int32_t* counts, cudaStream_t s,
-                       int tiles, bool two) {
+                       int tiles, bool two, const uint8_t* const* src, const int* src_pitch) {
     constexpr int CAP = kTileCap[FORM];
     const TileKernel<CAP>& kern = kernel_of<FORM>(ctx->cfg.nms_radius);
     const auto fn = kern.fn[ctx->cfg.score];
     TileCall<CAP> c;
-    std::memset(&c, 0, offsetof(TileCall<CAP>, tiles));
+    std::memset(&c, 0, offsetof(TileCall<CAP>, tiles) + sizeof(c.tiles[0]));
     size_t koff = 0, poff = ctx->group_pyr0;
     for (int i = 0; i < n; ++i) {
         FrameDesc& f = c.f[i];
@@ -85,6 +99,10 @@ vio_status detect_form(vio_ctx* ctx, const uint8_t* const* lev0, const int* pitc
         f.out = outs[i];
         f.lev[0] = const_cast<uint8_t*>(lev0[i]);
         f.pitch[0] = pitch0[i];
+        if (src && src[i]) {
+            f.src0 = src[i];
+            f.src0_pitch = src_pitch[i];
+        }
         koff += align_up((size_t)f.gw * f.gh, 16);
         for (int k = 1; k < levels; ++k) {
             f.pitch[k] = (int)align_up(f.w >> k, 128);
@@ -114,7 +132,7 @@ vio_status detect_form(vio_ctx* ctx, const uint8_t* const* lev0, const int* pitc
     c.n_frames = n;
     c.levels = levels;
     c.counts = counts;
-    const bool decode_launch = two || tiles > kLastTileDecodes;
+    const bool decode_launch = src || two || tiles > kLastTileDecodes;
     c.done = decode_launch ? nullptr : ctx->d_done;
     c.sums = ctx->d_sums;
     c.status = ctx->d_status;
@@ -151,7 +169,13 @@ vio_status detect_form(vio_ctx* ctx, const uint8_t* const* lev0, const int* pitc
             for (int i = 0; i < n; ++i) c.tiles[j * n + i + 1] = acc += tiles_of(dims[i], top - j, kern.tile_h);
         return launch_grid(fn, acc, kern.smem, dependent);
     };
-    if (!two) {
+    if (src) {
+        for (int i = 0; i < n; ++i) c.tiles[i + 1] = c.tiles[i] + pyr_plan(c.f[i], levels);
+        if ((st = launch_grid(pyramid_of<CAP>(levels), std::min(c.tiles[n], 8 * ctx->sm_count), 0, false)) != VIO_OK)
+            return st;
+        c.resident = levels - 1;
+        if ((st = launch_levels(levels - 1, levels, true)) != VIO_OK) return st;
+    } else if (!two) {
         if ((st = launch_levels(levels - 1, levels, false)) != VIO_OK) return st;
     } else {
         c.emit = std::min(levels - 1, 2);
@@ -183,7 +207,7 @@ namespace vio {
 
 vio_status detect_tiles(vio_ctx* ctx, const uint8_t* const* lev0, const int* pitch0, const vio_dims* dims, int n,
                         int thresh, int arc, int cell, int levels, int4* const* outs, int32_t* counts, cudaStream_t s,
-                        bool* done) {
+                        bool* done, const uint8_t* const* src, const int* src_pitch) {
     *done = false;
     // a pinned or tuned launch shape and stage times ask for the three kernels
     if (n > kTileCap[1] || ctx->cfg.profile || ctx->cfg.autotune || ctx->pinned_variant >= 0) return VIO_OK;
@@ -195,14 +219,22 @@ vio_status detect_tiles(vio_ctx* ctx, const uint8_t* const* lev0, const int* pit
         for (int k = 0; k < levels; ++k)
             for (int f = 0; f < 2; ++f) tiles[f] += tiles_of(dims[i], k, th[f]);
     }
+    if (src) {
+        if (tiles[1] > kFormTiles[1]) return VIO_OK;
+        *done = true;
+        return detect_form<1>(ctx, lev0, pitch0, dims, n, thresh, arc, cell, levels, outs, counts, s, tiles[1], false,
+                              src, src_pitch);
+    }
     const bool one = levels <= 3 && aligned;
     if (one && n <= kTileCap[0] && tiles[0] <= kFormTiles[0]) {
         *done = true;
-        return detect_form<0>(ctx, lev0, pitch0, dims, n, thresh, arc, cell, levels, outs, counts, s, tiles[0], false);
+        return detect_form<0>(ctx, lev0, pitch0, dims, n, thresh, arc, cell, levels, outs, counts, s, tiles[0], false,
+                              nullptr, nullptr);
     }
     if (tiles[1] <= (one ? kFormTiles[1] : kTwoStepTiles[aligned ? 0 : 1])) {
         *done = true;
-        return detect_form<1>(ctx, lev0, pitch0, dims, n, thresh, arc, cell, levels, outs, counts, s, tiles[1], !one);
+        return detect_form<1>(ctx, lev0, pitch0, dims, n, thresh, arc, cell, levels, outs, counts, s, tiles[1], !one,
+                              nullptr, nullptr);
     }
     return VIO_OK;
 }

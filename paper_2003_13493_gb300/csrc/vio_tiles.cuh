@@ -265,7 +265,19 @@ __global__ void __launch_bounds__(kConsumers, 5) tile_detect_kernel(const __grid
     }
 }
 
-// Decode of a call in two launches: one thread per cell, blocks of 256 cells of
+// Pyramids of frames that it also uploads (FrameDesc::src0: the device mapping
+// of host memory); blocks: prefix sums per frame, in tiles[].
+template <int L, int CAP>
+__global__ void __launch_bounds__(256) tile_pyramid_kernel(const __grid_constant__ TileCall<CAP> call) {
+    griddep_launch_dependents();
+    const int n = call.n_frames, blocks = call.tiles[n];
+    for (int b = blockIdx.x; b < blocks; b += gridDim.x) {
+        const int f = upper_index(call.tiles, n, b);
+        pyramid_block<L>(call.f[f], b - call.tiles[f]);
+    }
+}
+
+// Decode in a launch of its own: one thread per cell, blocks of 256 cells of
 // one frame (blocks: prefix sums per frame, in tiles[]).  A frame's count is
 // added up over its blocks in sums[], which the frame's last block hands over
 // and clears: the low half counts blocks, the high half cells.
