@@ -742,11 +742,14 @@ vio_status detect_in_groups(vio_ctx* ctx, const UploadPlan& plan, const uint8_t*
     for (int i = 0; i < n; ++i) lev0[i] = ctx->d_in + plan.off[i];
     struct Reset {
         vio_ctx* c;
+        bool failed;
         ~Reset() {
             c->group_pyr0 = 0;
             c->group_follows = false;
+            // no copy of a call that failed is left under way on a stream its caller cannot wait for
+            if (failed) cudaStreamSynchronize(c->copy_stream);
         }
-    } reset{ctx};
+    } reset{ctx, true};
     int copy = 0, copy_first = 0;  // the plan's current copy and its first frame
     for (int first = 0, g = 0; first < n; ++g) {
         size_t bytes = 0;
@@ -783,6 +786,7 @@ vio_status detect_in_groups(vio_ctx* ctx, const UploadPlan& plan, const uint8_t*
             return st;
         first = end;
     }
+    reset.failed = false;
     return VIO_OK;
 }
 

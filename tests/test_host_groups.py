@@ -74,3 +74,31 @@ def test_a_budget_that_held_one_call_holds_the_groups():
         lo, hi = (lo, mid) if works(mid, True) is not None else (mid, hi)
     a, b = works(hi, True), works(hi, False)
     assert b is not None and all(np.array_equal(x, y) for x, y in zip(a, b))
+
+
+def test_a_call_that_fails_within_its_groups_leaves_the_context_usable():
+    """The cell keys are a call's last buffer: just below the smallest budget a group fails after its copy began."""
+    imgs = [synth.make_frame(1280, 720, seed=i) for i in range(12)]
+    small = synth.make_frame(320, 240, seed=77)
+    frames, hold = layout(imgs, "ring")
+
+    def detector(budget):
+        return vio.Detector(max_frames=12, mem_budget_bytes=budget)
+
+    lo, hi = 1 << 20, 64 << 20
+    while hi - lo > 1024:
+        mid = (lo + hi) // 2
+        try:
+            det = detector(mid)
+            det.detect_host(frames, 15, 9, 32, 3)
+            det.close()
+            hi = mid
+        except vio.VioError:
+            lo = mid
+    det = detector(hi - 4096)
+    with pytest.raises(vio.VioError):
+        det.detect_host(frames, 15, 9, 32, 3)
+    outs, counts = det.detect_host([small], 15, 9, 32, 3)
+    want, c = oracle.detect(small, 15, 9, 32, 3)
+    assert np.array_equal(outs[0], want) and counts[0] == c
+    det.close()
