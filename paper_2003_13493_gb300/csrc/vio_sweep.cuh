@@ -173,6 +173,7 @@ __global__ void __launch_bounds__(kThreads, 3) fast_sweep_kernel(const uint8_t* 
             const int xw = xoff / 4;
             // levels >= 1: the run of even circle points that the shortest
             // arc needs; level 0, where few pixels pass at all: two compass points
+            // (32 4K frames, 8 settings: 821 us a call, 850 with the run on level 0 too)
             if (k > 0)
                 total = high_t ? coarse_and_compact<true, TH, 1>(img, queue, xw, k7, arc_min, warp, lane, row_lo,
                                                                               row_hi, vm, status)
