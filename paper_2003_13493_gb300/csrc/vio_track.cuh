@@ -200,17 +200,27 @@ __device__ __forceinline__ void window_store(const uint2 (&w)[kWinLoads], uint8_
     }
 }
 
-// A window at the right or lower border, or of a small image, byte by byte (a
-// lane per column); out of line, so that the loops stay short.
-__device__ __noinline__ void window_bytes(const Window& v, const uint8_t* img, int pitch, int lane, uint8_t* win) {
-    const int rows = min(kWinRows, v.h - v.y);
-    if (v.x + lane < v.w) {
-        const uint8_t* p = img + (size_t)v.y * pitch + v.x + lane;
-        uint8_t b[kWinRows];
+// One window, out of line so that the loops stay short: a track that has left
+// its window, and windows at the right or lower border or of a small image,
+// which come byte by byte (a lane per column).  A feature that never settles
+// (translation only, intensities that change) leaves its window again and again:
+// byte by byte everywhere, 100 such features took 53.8 us a call, with 8-byte loads
+// where they fit 43.3 (byte loads from memory in every iteration: 48.0).
+__device__ __noinline__ void window_fill(const Window& v, const uint8_t* img, int pitch, int lane, uint8_t* win) {
+    if (v.whole()) {
+        uint2 w[kWinLoads];
+        window_load(v, img, pitch, lane, w);
+        window_store(w, win, lane);
+    } else {
+        const int rows = min(kWinRows, v.h - v.y);
+        if (v.x + lane < v.w) {
+            const uint8_t* p = img + (size_t)v.y * pitch + v.x + lane;
+            uint8_t b[kWinRows];
 #pragma unroll
-        for (int r = 0; r < kWinRows; ++r) b[r] = r < rows ? p[(size_t)r * pitch] : (uint8_t)0;
+            for (int r = 0; r < kWinRows; ++r) b[r] = r < rows ? p[(size_t)r * pitch] : (uint8_t)0;
 #pragma unroll
-        for (int r = 0; r < kWinRows; ++r) win[r * kWinCols + lane] = b[r];
+            for (int r = 0; r < kWinRows; ++r) win[r * kWinCols + lane] = b[r];
+        }
     }
     __syncwarp();
 }
@@ -263,8 +273,8 @@ __device__ bool track_level(const TrackLevel& lv, float cx, float cy, TrackShare
         window_store(a, sh.prev, lane);
         window_store(b, sh.next, lane);
     } else {
-        window_bytes(wp, lv.prev, lv.pitch_prev, lane, sh.prev);
-        window_bytes(wn, lv.next, lv.pitch_next, lane, sh.next);
+        window_fill(wp, lv.prev, lv.pitch_prev, lane, sh.prev);
+        window_fill(wn, lv.next, lv.pitch_next, lane, sh.next);
     }
     __syncwarp();
 #pragma unroll
@@ -343,7 +353,7 @@ __device__ bool track_level(const TrackLevel& lv, float cx, float cy, TrackShare
         if (!wn.holds(c0, r0, P + 2)) {  // the track has left the window
             wn = Window::around(c0, r0, P + 2, lv.w, lv.h);
             __syncwarp();
-            window_bytes(wn, lv.next, lv.pitch_next, lane, sh.next);
+            window_fill(wn, lv.next, lv.pitch_next, lane, sh.next);
         }
         // this lane's samples: column xs, rows ys .. ys + NPX - 1 of the next image
         const float xs = o0 + (float)col + tx, ys = o1 + (float)row0 + ty;
