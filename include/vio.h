@@ -133,7 +133,8 @@ size_t vio_num_cells(int w, int h, int cell_size);
  *
  *   frames     host array of n_frames DEVICE pointers to uint8 frames.  A
  *              frame whose address is not 16-byte aligned or whose pitch is
- *              not a multiple of 16 is first copied into a context slot.
+ *              not a multiple of 16 is read by slower loads or staged in a
+ *              context slot by the pyramid kernel.
  *   dims       host array of n_frames vio_dims.
  *   thresh     0..255 (>= 1 when the context scores with MT, whose score
  *              would otherwise be 0 for a corner).
@@ -454,7 +455,7 @@ void vio_track_params_default(vio_track_params* p);
  *   prev, next  host arrays of n_pairs DEVICE pointers to uint8 frames; pair
  *               i has both frames of size dims[i] (pitch dims[i].pitch).
  *               Frames whose address or pitch is not a multiple of 16 are
- *               first copied into a context slot.
+ *               staged in a context slot by the pyramid kernel.
  *   pts         host array of n_pairs DEVICE pointers to float[2 * n_pts[i]]
  *               level-0 positions (x, y) in prev[i]
  *   n_pts       host int[n_pairs], each >= 0
