@@ -956,10 +956,12 @@ vio_status vio_create(vio_ctx** out, const vio_config* cfg_in) {
         vio_destroy(ctx);
         return s;
     };
+    if (cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking) != cudaSuccess)
+        return cleanup(VIO_ERR_CUDA);
     if (cudaMalloc(&ctx->d_call, ctx->call_cap) != cudaSuccess) return cleanup(VIO_ERR_OOM);
     constexpr size_t counter_bytes = 16 + (sizeof(uint64_t) + sizeof(int32_t)) * kTileCap[1];
     if (cudaMalloc(&ctx->d_counter, counter_bytes) != cudaSuccess) return cleanup(VIO_ERR_OOM);
-    if (cudaMemset(ctx->d_counter, 0, counter_bytes) != cudaSuccess) return cleanup(VIO_ERR_CUDA);
+    if (clear_now(ctx, ctx->d_counter, counter_bytes) != cudaSuccess) return cleanup(VIO_ERR_CUDA);
     ctx->d_sums = reinterpret_cast<uint64_t*>(ctx->d_counter + 4);
     ctx->d_done = reinterpret_cast<int32_t*>(ctx->d_sums + kTileCap[1]);
     if (cudaHostAlloc(&ctx->h_status, 64, cudaHostAllocMapped) != cudaSuccess) return cleanup(VIO_ERR_OOM);
@@ -975,8 +977,6 @@ vio_status vio_create(vio_ctx** out, const vio_config* cfg_in) {
     if (cudaEventCreateWithFlags(&ctx->last_ev, cudaEventDisableTiming) != cudaSuccess) return cleanup(VIO_ERR_CUDA);
     for (auto& e : ctx->stage_ev)
         if (cudaEventCreate(&e) != cudaSuccess) return cleanup(VIO_ERR_CUDA);
-    if (cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking) != cudaSuccess)
-        return cleanup(VIO_ERR_CUDA);
     ctx->bytes_in_use = ctx->call_cap;
     *out = ctx;
     return VIO_OK;

@@ -126,7 +126,7 @@ struct vio_ctx {
     size_t h_out_cap = 0;
 
     cudaEvent_t stage_ev[4] = {nullptr, nullptr, nullptr, nullptr};
-    cudaStream_t capture_stream = nullptr;
+    cudaStream_t capture_stream = nullptr;  // the context's own: graphs are captured and buffers cleared on it
     cudaEvent_t last_ev = nullptr;
     cudaStream_t last_stream = nullptr;
     bool have_last = false;
@@ -193,6 +193,14 @@ inline vio_status fail(vio_ctx* c, vio_status s, const std::string& msg) {
         }                                                                                     \
     } while (0)
 
+// Clears device memory and waits for it, on a stream of the context's own: the
+// caller's stream may be one that the default stream does not order itself with,
+// and work queued on the default stream is none of the call's business.
+inline cudaError_t clear_now(vio_ctx* ctx, void* p, size_t bytes) {
+    const cudaError_t e = cudaMemsetAsync(p, 0, bytes, ctx->capture_stream);
+    return e != cudaSuccess ? e : cudaStreamSynchronize(ctx->capture_stream);
+}
+
 // Grows a resident buffer to `need` bytes.  Growing waits for the device
 // (the old buffer may still be in use), so buffers grow geometrically.
 inline vio_status grow(vio_ctx* ctx, void** p, size_t* cap, size_t need, bool zero) {
@@ -212,7 +220,7 @@ inline vio_status grow(vio_ctx* ctx, void** p, size_t* cap, size_t need, bool ze
         *cap = 0;
     }
     VIO_CK(cudaMalloc(p, want));
-    if (zero) VIO_CK(cudaMemset(*p, 0, want));
+    if (zero) VIO_CK(clear_now(ctx, *p, want));
     *cap = want;
     ctx->bytes_in_use += want;
     return VIO_OK;
