@@ -829,6 +829,8 @@ vio_status detect_from_host(vio_ctx* ctx, const uint8_t* const* host_frames, con
         ctx->pinned_variant < 0)
         return detect_in_groups(ctx, plan, host_frames, dims, n, thresh, arc, cell, levels, outs, d_counts, s);
     if (!any_up) std::fill(skip.begin(), skip.end(), false);
+    // the context's previous call may still read frames staged in this buffer
+    if (ctx->have_last && ctx->last_stream != s) VIO_CK(cudaStreamWaitEvent(s, ctx->last_ev, 0));
     if ((st = enqueue_upload(ctx, plan, ctx->d_in, s, &skip)) != VIO_OK) return st;
     Upload up;
     if (any_up) {

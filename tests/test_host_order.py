@@ -171,3 +171,26 @@ def test_cleared_buffers_are_ready_on_any_stream(host, sizes):
             if c < first:
                 assert ordered(log, c, first), (log[c], hex(s))
     assert clears[0] < clears[1] < launches[S1] < clears[2] < launches[S2]
+
+
+@pytest.mark.parametrize("before", ["sweep", "detect"])
+@pytest.mark.parametrize("sizes", [[(640, 480)], [(1920, 1080)] * 4], ids=["one copy", "groups"])
+def test_an_upload_waits_for_the_frames_staged_before_it(host, before, sizes):
+    """Unaligned device frames and host frames share the context's input buffer: a host call's copies follow the
+    kernels of an earlier call on another stream that read it."""
+    h = host(max_frames=64)
+    unaligned = [(1921, 1081)] * 30
+    assert h.detect_host([(1920, 1080)] * 32, S2) == 0  # the buffer is large enough from here on
+    h.log(clear=True)
+    if before == "sweep":
+        assert h.sweep(unaligned, S1, align=False) == 0
+    else:
+        assert h.detect(unaligned, S1, align=False) == 0
+    assert h.detect_host(sizes, S2) == 0
+    log = h.log()
+    assert not [e for e in log if e[0] == "malloc" and int(e[3]) > 4 << 20]
+    launch = max(i for i, e in enumerate(log) if e[0] == "launch" and int(e[1], 16) == S1)
+    copies = [i for i, e in enumerate(log) if e[0] == "copy" and i > launch and int(e[4]) > 200_000]
+    assert copies
+    for c in copies:
+        assert ordered(log, launch, c), log[c]
