@@ -725,10 +725,29 @@ vio_status detect_in_groups(vio_ctx* ctx, const UploadPlan& plan, const uint8_t*
             pyr += align_up(align_up(dims[i].w >> k, 128) * (size_t)(dims[i].h >> k), 256);
         pyr_at[i + 1] = pyr;
     }
-    // room for all groups' levels, so that no group grows the buffer
+    // the groups' ends, and the cell keys of the group that needs most
+    const size_t want = std::max(kGroupMin, total / 6 + 1);
+    std::vector<int> group_end;
+    size_t keys = 0;
+    for (int i = 0; i < n;) {
+        size_t bytes = 0, k = 0;
+        const int first = i;
+        while (i < n && ((int)group_end.size() == kMaxGroups - 1 || i == first ||
+                         bytes + (size_t)dims[i].w * dims[i].h <= want)) {
+            bytes += (size_t)dims[i].w * dims[i].h;
+            k += align_up(vio_num_cells(dims[i].w, dims[i].h, cell), 16);
+            ++i;
+        }
+        keys = std::max(keys, k);
+        group_end.push_back(i);
+    }
+    // room for all groups' levels and for any group's keys: no group grows a
+    // buffer, and a call over the budget ends before any work is enqueued
+    const void* keys0 = ctx->d_keys;
     const void* pyr0 = ctx->d_pyr;
+    if ((st = grow(ctx, (void**)&ctx->d_keys, &ctx->keys_cap, keys * 8, true)) != VIO_OK) return st;
     if ((st = grow(ctx, (void**)&ctx->d_pyr, &ctx->pyr_cap, std::max<size_t>(pyr, 256), false)) != VIO_OK) return st;
-    if (pyr0 != ctx->d_pyr) ctx->map_cache.clear();
+    if (keys0 != ctx->d_keys || pyr0 != ctx->d_pyr) ctx->map_cache.clear();
     if (!ctx->copy_stream) VIO_CK(cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking));
     for (auto& e : ctx->group_ev)
         if (!e) VIO_CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
@@ -738,56 +757,57 @@ vio_status detect_in_groups(vio_ctx* ctx, const UploadPlan& plan, const uint8_t*
     VIO_CK(cudaStreamWaitEvent(ctx->copy_stream, ctx->group_ev[0], 0));
     if (ctx->have_last) VIO_CK(cudaStreamWaitEvent(ctx->copy_stream, ctx->last_ev, 0));
     std::vector<const uint8_t*> lev0(n);
-    const size_t want = std::max(kGroupMin, total / 6 + 1);
     for (int i = 0; i < n; ++i) lev0[i] = ctx->d_in + plan.off[i];
     struct Reset {
         vio_ctx* c;
-        bool failed;
         ~Reset() {
             c->group_pyr0 = 0;
             c->group_follows = false;
-            // no copy of a call that failed is left under way on a stream its caller cannot wait for
-            if (failed) cudaStreamSynchronize(c->copy_stream);
         }
-    } reset{ctx, true};
-    int copy = 0, copy_first = 0;  // the plan's current copy and its first frame
-    for (int first = 0, g = 0; first < n; ++g) {
-        size_t bytes = 0;
-        int end = first;
-        while (end < n && (g == kMaxGroups - 1 || end == first || bytes + (size_t)dims[end].w * dims[end].h <= want)) {
-            bytes += (size_t)dims[end].w * dims[end].h;
-            ++end;
-        }
-        // the group's part of the plan: whole copies, and its frames of a span
-        for (int i = first; i < end;) {
-            const UploadPlan::Copy& cp = plan.copies[copy];
-            const int copy_end = copy_first + plan.span_len[copy_first], j = std::min(end, copy_end);
-            if (cp.w == 0) {
-                const vio_dims& d = dims[j - 1];
-                const size_t part = (size_t)(host_frames[j - 1] + (size_t)d.pitch * (d.h - 1) + d.w - host_frames[i]);
-                VIO_CK(cudaMemcpyAsync(ctx->d_in + plan.off[i], host_frames[i], part, cudaMemcpyHostToDevice,
-                                       ctx->copy_stream));
-            } else {
-                VIO_CK(cudaMemcpy2DAsync(ctx->d_in + cp.dst, cp.dpitch, cp.src, cp.spitch, cp.w, cp.h,
-                                         cudaMemcpyHostToDevice, ctx->copy_stream));
+    } reset{ctx};
+    const auto run_groups = [&]() -> vio_status {
+        int copy = 0, copy_first = 0;  // the plan's current copy and its first frame
+        for (int first = 0, g = 0; first < n; ++g) {
+            const int end = group_end[g];
+            // the group's part of the plan: whole copies, and its frames of a span
+            for (int i = first; i < end;) {
+                const UploadPlan::Copy& cp = plan.copies[copy];
+                const int copy_end = copy_first + plan.span_len[copy_first], j = std::min(end, copy_end);
+                if (cp.w == 0) {
+                    const vio_dims& d = dims[j - 1];
+                    const size_t part = (size_t)(host_frames[j - 1] + (size_t)d.pitch * (d.h - 1) + d.w - host_frames[i]);
+                    VIO_CK(cudaMemcpyAsync(ctx->d_in + plan.off[i], host_frames[i], part, cudaMemcpyHostToDevice,
+                                           ctx->copy_stream));
+                } else {
+                    VIO_CK(cudaMemcpy2DAsync(ctx->d_in + cp.dst, cp.dpitch, cp.src, cp.spitch, cp.w, cp.h,
+                                             cudaMemcpyHostToDevice, ctx->copy_stream));
+                }
+                i = j;
+                if (j == copy_end) {
+                    copy_first = copy_end;
+                    ++copy;
+                }
             }
-            i = j;
-            if (j == copy_end) {
-                copy_first = copy_end;
-                ++copy;
-            }
+            VIO_CK(cudaEventRecord(ctx->group_ev[1 + g], ctx->copy_stream));
+            VIO_CK(cudaStreamWaitEvent(s, ctx->group_ev[1 + g], 0));
+            ctx->group_pyr0 = pyr_at[first];
+            ctx->group_follows = first > 0;
+            if ((st = detect_impl(ctx, lev0.data() + first, plan.pitch.data() + first, dims + first, end - first, thresh,
+                                  arc, cell, levels, outs + first, d_counts ? d_counts + first : nullptr, s)) != VIO_OK)
+                return st;
+            first = end;
         }
-        VIO_CK(cudaEventRecord(ctx->group_ev[1 + g], ctx->copy_stream));
-        VIO_CK(cudaStreamWaitEvent(s, ctx->group_ev[1 + g], 0));
-        ctx->group_pyr0 = pyr_at[first];
-        ctx->group_follows = first > 0;
-        if ((st = detect_impl(ctx, lev0.data() + first, plan.pitch.data() + first, dims + first, end - first, thresh,
-                              arc, cell, levels, outs + first, d_counts ? d_counts + first : nullptr, s)) != VIO_OK)
-            return st;
-        first = end;
-    }
-    reset.failed = false;
-    return VIO_OK;
+        return VIO_OK;
+    };
+    st = run_groups();
+    if (st == VIO_OK) return st;
+    // The call is a synchronous one: when it returns an error no copy still reads
+    // the caller's frames, no kernel of an earlier group still writes records, and
+    // what those kernels report is this call's error, not the next one's.
+    cudaStreamSynchronize(ctx->copy_stream);
+    cudaStreamSynchronize(s);
+    const vio_status device_st = take_status(ctx);
+    return device_st != VIO_OK ? device_st : st;
 }
 
 }  // namespace

@@ -194,3 +194,41 @@ def test_an_upload_waits_for_the_frames_staged_before_it(host, before, sizes):
     assert copies
     for c in copies:
         assert ordered(log, launch, c), log[c]
+
+
+@pytest.mark.parametrize("op,nth", [("launch", 3), ("launch", 5), ("copy", 3)])
+def test_a_grouped_call_that_fails_leaves_nothing_in_flight(host, op, nth):
+    """The caller of a synchronous call may free its buffers when it returns, also with an error: no kernel of an
+    earlier group still writes records, and no copy still reads frames."""
+    h = host(max_frames=64)
+    sizes = [(1280, 720)] * 24
+    assert h.detect_host(sizes, S1) == 0
+    h.log(clear=True)
+    h.lib.fake_fail(op.encode(), nth)
+    assert h.detect_host(sizes, S1) == 3
+    log = h.log(clear=True)
+    work = [i for i, e in enumerate(log) if e[0] in ("launch", "copy")]
+    assert [e for e in log if e[0] == "launch"] and len({log[i][1] for i in work}) == 2
+    end = len(log)
+    for i in work:
+        assert ordered(log + [["host", "-"]], i, end), log[i]
+    assert h.detect_host(sizes, S1) == 0
+
+
+def test_a_grouped_call_over_the_budget_starts_nothing(host):
+    """Every buffer that any group needs is there before the first group begins, so a budget that is too small by
+    the keys of a late, larger group is found before any work is enqueued."""
+    small, large = [(1280, 720)] * 12, [(3840, 2160)] * 3
+
+    def attempt(budget):
+        h = host(max_frames=64, mem_budget_bytes=budget)
+        h.log(clear=True)
+        return h.detect_host(small + large, S1, cell=32), h.log(clear=True)
+
+    lo, hi = 1 << 20, 256 << 20  # the smallest budget that works
+    while hi - lo > 256:
+        mid = (lo + hi) // 2
+        lo, hi = (lo, mid) if attempt(mid)[0] == 0 else (mid, hi)
+    for budget in (lo, lo - 4096, lo - 65536):
+        status, log = attempt(budget)
+        assert status == 2 and not [e for e in log if e[0] in ("launch", "copy")], budget
