@@ -194,20 +194,30 @@ struct PyrRow {
     }
 };
 
+// Thread `thread`'s chunk in block `block` of a frame.
+struct PyrChunk {
+    int tx, ty;  // column and row of chunks
+};
+__host__ __device__ __forceinline__ PyrChunk pyr_chunk(const FrameDesc& fd, int block, int thread) {
+    const int cx = fd.pyr_cx;
+    // chunk number = ty * cx + tx.  The product with ceil(2^32 / cx) gives the
+    // row of the block's first chunk or one more (a frame has at most 2^24
+    // chunks), the division of a thread's chunk alike.
+    const auto divide = [&](int v) {
+        const int q = (int)(((uint64_t)(uint32_t)v * fd.pyr_magic) >> 32);
+        return q * cx > v ? q - 1 : q;
+    };
+    const int first = block * 256, row = divide(first);
+    const int off = first - row * cx + thread, down = divide(off);
+    return {off - down * cx, row + down};
+}
+
 // Block `block` of a frame: 256 chunks, one per thread.
 template <int L>
 __device__ __forceinline__ void pyramid_block(const FrameDesc& fd, int block) {
     constexpr int B = pyr_rows(L);
-    const int cx = fd.pyr_cx;
-    // chunk number = ty * cx + tx.  The product with ceil(2^32 / cx) gives
-    // the row of the block's first chunk or one more (at most 2^24 chunks
-    // of at most 2^12 per row), and exactly the row of a number below 2^13.
-    const int first = block * 256;
-    int row = (int)__umulhi((uint32_t)first, fd.pyr_magic);
-    if (row * cx > first) --row;
-    const int off = first - row * cx + (int)threadIdx.x;
-    const int down = (int)__umulhi((uint32_t)off, fd.pyr_magic);
-    const int tx = off - down * cx, ty = row + down;
+    const PyrChunk c = pyr_chunk(fd, block, (int)threadIdx.x);
+    const int tx = c.tx, ty = c.ty;
     const int W = fd.w, H = fd.h, x0 = tx * 16, y0 = ty * B;
     if (x0 >= W || y0 >= H) return;
     const bool upload = fd.src0 != nullptr;

@@ -19,8 +19,7 @@ OUT = os.path.join(HERE, "_build")
 def build_host_library():
     """The library's host code over the fake runtime (device code is compiled but never runs)."""
     lib = os.path.join(OUT, "libvio_host.so")
-    fake = os.path.join(HERE, "fake_cuda", "runtime.cpp")
-    sources = sorted(glob.glob(os.path.join(build.CSRC, "*.cu"))) + [fake]
+    sources = sorted(glob.glob(os.path.join(build.CSRC, "*.cu")) + glob.glob(os.path.join(HERE, "fake_cuda", "*.c*")))
     deps = sources + glob.glob(os.path.join(build.CSRC, "*.*h")) + glob.glob(os.path.join(build.INCLUDE, "*.h"))
     if os.path.exists(lib) and all(os.path.getmtime(p) < os.path.getmtime(lib) for p in deps):
         return lib
