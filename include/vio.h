@@ -47,6 +47,11 @@
  *     context owns its resident pyramid, cell-key, descriptor and
  *     tensor-map buffers; they grow on demand up to mem_budget_bytes
  *     (VIO_ERR_OOM past it).
+ *   - Stream capture: a context's calls are not for capture (in global and
+ *     thread-local mode they return VIO_ERR_CUDA and the capture is invalid):
+ *     a graph launched later would use resident buffers that a larger call
+ *     may have replaced.
+ *     vio_detect_noalloc can be captured.
  *   - Threading: a context serves one host thread at a time.
  */
 #ifndef VIO_H_

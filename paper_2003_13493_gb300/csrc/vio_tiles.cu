@@ -211,6 +211,14 @@ vio_status detect_tiles(vio_ctx* ctx, const uint8_t* const* lev0, const int* pit
     *done = false;
     // a pinned or tuned launch shape and stage times ask for the three kernels
     if (n > kTileCap[1] || ctx->cfg.profile || ctx->cfg.autotune || ctx->pinned_variant >= 0) return VIO_OK;
+    // So does a stream that is being captured: their call block keeps a detection
+    // out of a graph, whose later launches would use resident buffers that may have
+    // been given back (vio_detect_noalloc is the call to capture).
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return VIO_OK;
+    }
     int tiles[2] = {0, 0};
     const int th[2] = {kernel_of<0>(ctx->cfg.nms_radius).tile_h, kernel_of<1>(ctx->cfg.nms_radius).tile_h};
     bool aligned = true;

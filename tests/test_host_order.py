@@ -231,3 +231,18 @@ def test_a_grouped_call_over_the_budget_starts_nothing(host):
     for budget in (lo, lo - 4096, lo - 65536):
         status, log = attempt(budget)
         assert status == 2 and not [e for e in log if e[0] in ("launch", "copy")], budget
+
+
+@pytest.mark.parametrize("sizes,align", [([(752, 480)], True), ([(1280, 720)] * 16, True), ([(641, 480)] * 4, False)])
+def test_a_captured_stream_takes_the_persistent_kernels(host, sizes, align):
+    """Inside a caller's stream capture a detection is refused: a graph replayed later would use resident buffers
+    that have been given back when a larger call grew them.  The kernels of small calls are no way around that."""
+    h = host(max_frames=64)
+    for _ in range(2):
+        assert h.detect(sizes, S1, align=align) == 0
+    assert any("tile_detect" in e[2] for e in h.log(clear=True) if e[0] == "launch")
+    h.lib.fake_capturing(S1, 1)
+    assert h.detect(sizes, S1, align=align) == 3
+    assert not [e for e in h.log() if e[0] == "launch"]
+    h.lib.fake_capturing(None, 0)
+    assert h.detect(sizes, S1, align=align) == 0
