@@ -271,17 +271,27 @@ vio_status vio_selftest_timeout(vio_ctx* ctx, uint32_t limit_us);
  * fit), nms_radius the NMS window the variant was built for, cell_size the
  * grid cell size of the detection.
  *
+ * Small and middling calls of a context with nothing pinned, autotune off and
+ * profiling off take another kernel, one CTA per tile, which is none of the
+ * variants; a pinned, tuning or profiling context uses the variants for every
+ * call.
+ *
  * vio_get_tuning reports the configuration of the context's most recent
  * detection (cta_per_sm resolved to the count launched; cell_size the one
- * used, also when vio_detect was given cell_size 0).  vio_set_tuning pins a
- * variant and a CTA count for later calls (NULL unpins; VIO_ERR_INVALID_ARG
- * if the variant is not one of the built ones, was built for another NMS
- * radius than the context's, or cta_per_sm is outside 0..4); its tile_w,
- * tile_h, nms_radius and cell_size fields are ignored.  With autotune on and
- * nothing pinned, the first vio_detect of a batch shape times every
- * combination of the radius's variants, 2 to 4 CTAs per SM (as far as they
- * fit) and, when cell_size is 0, cells of 32 and 64, and keeps the fastest
- * for that shape; vio_autotune_log returns what that run timed.
+ * used, also when vio_detect was given cell_size 0).  After a call of the
+ * tile kernel cta_per_sm is 0, tile_h that kernel's and variant the one that
+ * larger calls use; pinning that means that variant's persistent launch.
+ *
+ * vio_set_tuning pins a variant and a CTA count for later calls (NULL unpins;
+ * VIO_ERR_INVALID_ARG if the variant is not one of the built ones, was built
+ * for another NMS radius than the context's, or cta_per_sm is outside 0..4);
+ * its tile_w, tile_h, nms_radius and cell_size fields are ignored.  With
+ * autotune on and nothing pinned, the first vio_detect of a batch shape times
+ * every combination of the radius's variants, 2 to 4 CTAs per SM (as far as
+ * they fit) and, when cell_size is 0, cells of 32 and 64, and keeps the
+ * fastest of these for that shape (a small call can be faster untuned: the
+ * tile kernel is not among them); vio_autotune_log returns what that run
+ * timed.
  */
 typedef struct {
     int tile_w, tile_h, cta_per_sm, variant, nms_radius, cell_size;

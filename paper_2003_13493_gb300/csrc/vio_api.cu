@@ -557,6 +557,7 @@ vio_status launch(vio_ctx* ctx, int variant, const uint8_t* const* lev0, const i
     // a sweep's launch shape is fixed: the CTAs per SM its registers and
     // shared memory allow
     ctx->last_ctas = sweep ? ctx->grid_sweep / ctx->sm_count : (ctas > 0 ? std::min(ctas, occ) : occ);
+    ctx->last_tile_h = 0;
     ctx->last_cell = cell;
     return VIO_OK;
 }
@@ -1278,6 +1279,7 @@ vio_status vio_get_tuning(const vio_ctx* ctx, vio_tuning* out) {
     if (!ctx || !out) return VIO_ERR_INVALID_ARG;
     const int vi = ctx->pinned_variant >= 0 ? ctx->pinned_variant : ctx->last_variant;
     vio_variant(vi, out);
+    if (ctx->pinned_variant < 0 && ctx->last_tile_h > 0) out->tile_h = ctx->last_tile_h;
     out->cta_per_sm = ctx->last_ctas;
     out->cell_size = ctx->last_cell;
     return VIO_OK;

@@ -148,7 +148,8 @@ struct vio_ctx {
     int pinned_variant = -1;
     int pinned_ctas = 0;
     int last_variant = 0;
-    int last_ctas = 0;                     // CTAs per SM of the last launch (resolved)
+    int last_ctas = 0;                     // CTAs per SM of the last launch (resolved); 0: the tile kernel's
+    int last_tile_h = 0;                   // tile height of the tile kernel's last launch; 0: the variant's
     int last_cell = 0;                     // cell size of the last detection
     // levels of the most recent detection call, for vio_copy_level
     std::vector<std::array<const uint8_t*, vio::kMaxLevels>> last_lev;

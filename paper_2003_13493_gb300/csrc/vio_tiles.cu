@@ -196,7 +196,8 @@ vio_status detect_form(vio_ctx* ctx, const uint8_t* const* lev0, const int* pitc
     ctx->have_last = true;
     remember_levels(ctx, c.f, dims, n, levels);
     ctx->last_variant = ctx->default_variant;
-    ctx->last_ctas = 1;
+    ctx->last_ctas = 0;
+    ctx->last_tile_h = kern.tile_h;
     ctx->last_cell = cell;
     return VIO_OK;
 }
