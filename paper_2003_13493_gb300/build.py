@@ -25,7 +25,7 @@ def _sources() -> list[str]:
 
 
 def _deps() -> list[str]:
-    return _sources() + sorted(glob.glob(os.path.join(CSRC, "*.cuh"))) + \
+    return _sources() + sorted(glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h"))) + \
         sorted(glob.glob(os.path.join(INCLUDE, "*.h")))
 
 
