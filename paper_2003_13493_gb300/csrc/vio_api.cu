@@ -424,8 +424,7 @@ vio_status launch(vio_ctx* ctx, int variant, const uint8_t* const* lev0, const i
     if ((st = grow(ctx, (void**)&ctx->d_pyr, &ctx->pyr_cap, std::max<size_t>(poff, 256), false)) != VIO_OK) return st;
     if (keys0 != ctx->d_keys || pyr0 != ctx->d_pyr) ctx->map_cache.clear();
 
-    // order against work of this context on another stream
-    if (ctx->have_last && ctx->last_stream != s) VIO_CK(cudaStreamWaitEvent(s, ctx->last_ev, 0));
+    VIO_CK(follow_context(ctx, s));
     const int slot = ctx->ring_pos;
     ctx->ring_pos = (ctx->ring_pos + 1) % ctx->ring;
     VIO_CK(cudaEventSynchronize(ctx->ring_ev[slot]));
@@ -549,9 +548,7 @@ vio_status launch(vio_ctx* ctx, int variant, const uint8_t* const* lev0, const i
     } else if ((st = enqueue_kernels(ctx, variant, levels, s, pyramid, ctas)) != VIO_OK) {
         return st;
     }
-    VIO_CK(cudaEventRecord(ctx->last_ev, s));
-    ctx->last_stream = s;
-    ctx->have_last = true;
+    VIO_CK(mark_last(ctx, s));
     int occ = 1;
     if (!sweep) VIO_CK_STATUS(fused_occupancy(ctx, variant, &occ));
     // a sweep's launch shape is fixed: the CTAs per SM its registers and
@@ -979,12 +976,13 @@ vio_status vio_create(vio_ctx** out, const vio_config* cfg_in) {
         vio_destroy(ctx);
         return s;
     };
-    if (cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking) != cudaSuccess)
+    if (cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ctx->clear_ev, cudaEventDisableTiming) != cudaSuccess)
         return cleanup(VIO_ERR_CUDA);
     if (cudaMalloc(&ctx->d_call, ctx->call_cap) != cudaSuccess) return cleanup(VIO_ERR_OOM);
     constexpr size_t counter_bytes = 16 + (sizeof(uint64_t) + sizeof(int32_t)) * kTileCap[1];
     if (cudaMalloc(&ctx->d_counter, counter_bytes) != cudaSuccess) return cleanup(VIO_ERR_OOM);
-    if (clear_now(ctx, ctx->d_counter, counter_bytes) != cudaSuccess) return cleanup(VIO_ERR_CUDA);
+    if (clear_buffer(ctx, ctx->d_counter, counter_bytes) != cudaSuccess) return cleanup(VIO_ERR_CUDA);
     ctx->d_sums = reinterpret_cast<uint64_t*>(ctx->d_counter + 4);
     ctx->d_done = reinterpret_cast<int32_t*>(ctx->d_sums + kTileCap[1]);
     if (cudaHostAlloc(&ctx->h_status, 64, cudaHostAllocMapped) != cudaSuccess) return cleanup(VIO_ERR_OOM);
@@ -1031,6 +1029,7 @@ vio_status vio_destroy(vio_ctx* ctx) {
     for (auto& e : ctx->ring_ev)
         if (e) cudaEventDestroy(e);
     if (ctx->last_ev) cudaEventDestroy(ctx->last_ev);
+    if (ctx->clear_ev) cudaEventDestroy(ctx->clear_ev);
     for (auto& e : ctx->stage_ev)
         if (e) cudaEventDestroy(e);
     if (ctx->capture_stream) cudaStreamDestroy(ctx->capture_stream);

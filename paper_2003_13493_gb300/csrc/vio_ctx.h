@@ -130,6 +130,8 @@ struct vio_ctx {
     cudaEvent_t last_ev = nullptr;
     cudaStream_t last_stream = nullptr;
     bool have_last = false;
+    cudaEvent_t clear_ev = nullptr;         // after the latest clear of a buffer (clear_buffer)
+    bool clear_pending = false;             // no call has followed it yet
 
     // one graph per (variant, levels, CTAs per SM): every batch shape replays
     // it; CTAs per SM 0 = as many as fit
@@ -194,12 +196,39 @@ inline vio_status fail(vio_ctx* c, vio_status s, const std::string& msg) {
         }                                                                                     \
     } while (0)
 
-// Clears device memory and waits for it, on a stream of the context's own: the
-// caller's stream may be one that the default stream does not order itself with,
-// and work queued on the default stream is none of the call's business.
-inline cudaError_t clear_now(vio_ctx* ctx, void* p, size_t bytes) {
-    const cudaError_t e = cudaMemsetAsync(p, 0, bytes, ctx->capture_stream);
-    return e != cudaSuccess ? e : cudaStreamSynchronize(ctx->capture_stream);
+// Clears device memory on a stream of the context's own, for kernels enqueued
+// after follow_context: the default stream is not ordered with a caller's
+// non-blocking stream, and what is queued on it is none of the call's business.
+// (Waiting here instead costs a context's first call 10 us.)
+inline cudaError_t clear_buffer(vio_ctx* ctx, void* p, size_t bytes) {
+    cudaError_t e = cudaMemsetAsync(p, 0, bytes, ctx->capture_stream);
+    if (e == cudaSuccess) e = cudaEventRecord(ctx->clear_ev, ctx->capture_stream);
+    if (e == cudaSuccess) ctx->clear_pending = true;
+    return e;
+}
+
+// Orders `s` after the context's work on another stream and after its clears;
+// to be followed by mark_last once the call's work is enqueued.  (A call that fails
+// in between leaves its clears pending for the next one.)
+inline cudaError_t follow_context(vio_ctx* ctx, cudaStream_t s) {
+    cudaError_t e = cudaSuccess;
+    if (ctx->have_last && ctx->last_stream != s) e = cudaStreamWaitEvent(s, ctx->last_ev, 0);
+    if (e != cudaSuccess || !ctx->clear_pending) return e;
+    // (a capture cannot wait for work outside it: where one is allowed, the host does)
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    e = cudaStreamIsCapturing(s, &capture);
+    if (e != cudaSuccess) return e;
+    return capture == cudaStreamCaptureStatusNone ? cudaStreamWaitEvent(s, ctx->clear_ev, 0)
+                                                  : cudaEventSynchronize(ctx->clear_ev);
+}
+
+inline cudaError_t mark_last(vio_ctx* ctx, cudaStream_t s) {
+    const cudaError_t e = cudaEventRecord(ctx->last_ev, s);
+    if (e != cudaSuccess) return e;
+    ctx->last_stream = s;
+    ctx->have_last = true;
+    ctx->clear_pending = false;  // last_ev follows them
+    return e;
 }
 
 // Grows a resident buffer to `need` bytes.  Growing waits for the device
@@ -221,7 +250,7 @@ inline vio_status grow(vio_ctx* ctx, void** p, size_t* cap, size_t need, bool ze
         *cap = 0;
     }
     VIO_CK(cudaMalloc(p, want));
-    if (zero) VIO_CK(clear_now(ctx, *p, want));
+    if (zero) VIO_CK(clear_buffer(ctx, *p, want));
     *cap = want;
     ctx->bytes_in_use += want;
     return VIO_OK;

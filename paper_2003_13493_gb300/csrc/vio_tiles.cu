@@ -140,8 +140,7 @@ vio_status detect_form(vio_ctx* ctx, const uint8_t* const* lev0, const int* pitc
         const uint64_t d = (uint64_t)(cell >> k);
         c.cell_magic[k] = (uint32_t)(((1ull << 32) + d - 1) / d);
     }
-    // order against work of this context on another stream
-    if (ctx->have_last && ctx->last_stream != s) VIO_CK(cudaStreamWaitEvent(s, ctx->last_ev, 0));
+    VIO_CK(follow_context(ctx, s));
     if (!ctx->tile_ready[FORM]) {
         VIO_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kern.smem));
         ctx->tile_ready[FORM] = true;
@@ -191,9 +190,7 @@ vio_status detect_form(vio_ctx* ctx, const uint8_t* const* lev0, const int* pitc
         for (int i = 0; i < n; ++i) c.tiles[i + 1] = c.tiles[i] + (c.f[i].gw * c.f[i].gh + 255) / 256;
         if ((st = launch_grid(tile_decode_kernel<CAP>, c.tiles[n], 0, true)) != VIO_OK) return st;
     }
-    VIO_CK(cudaEventRecord(ctx->last_ev, s));
-    ctx->last_stream = s;
-    ctx->have_last = true;
+    VIO_CK(mark_last(ctx, s));
     remember_levels(ctx, c.f, dims, n, levels);
     ctx->last_variant = ctx->default_variant;
     ctx->last_ctas = 0;

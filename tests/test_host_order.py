@@ -172,6 +172,29 @@ def test_cleared_buffers_are_ready_on_any_stream(host, sizes):
     assert clears[0] < clears[1] < launches[S1] < clears[2] < launches[S2]
 
 
+@pytest.mark.parametrize("small", [[(640, 480)], [(160, 120)] * 70], ids=["tiles", "persistent"])
+def test_a_clear_outlives_the_call_that_asked_for_it(host, small):
+    """A call that grows the keys and then fails has enqueued nothing that a later call, on another stream, could wait
+    for but the clear itself."""
+    large = [(1920, 1080)] * 60
+
+    def attempt(budget):
+        h = host(max_frames=128, mem_budget_bytes=budget)
+        h.log(clear=True)
+        return h, h.detect(large, S1)
+
+    lo, hi = 1 << 20, 256 << 20  # the smallest budget that works
+    while hi - lo > 4096:
+        mid = (lo + hi) // 2
+        lo, hi = (lo, mid) if attempt(mid)[1] == 0 else (mid, hi)
+    h, status = attempt(lo - 65536)  # the keys fit, the pyramid does not
+    clear = next(i for i, e in enumerate(h.log()) if e[0] == "memset")
+    assert status == 2 and not [e for e in h.log() if e[0] == "launch"]
+    assert h.detect(small, S2) == 0
+    log = h.log()
+    assert ordered(log, clear, next(i for i, e in enumerate(log) if e[0] == "launch"))
+
+
 @pytest.mark.parametrize("before", ["sweep", "detect"])
 @pytest.mark.parametrize("sizes", [[(640, 480)], [(1920, 1080)] * 4], ids=["one copy", "groups"])
 def test_an_upload_waits_for_the_frames_staged_before_it(host, before, sizes):
