@@ -420,8 +420,8 @@ vio_status launch(vio_ctx* ctx, int variant, const uint8_t* const* lev0, const i
     const void* keys0 = ctx->d_keys;
     const void* pyr0 = ctx->d_pyr;
     const int n_set = sweep ? sweep->n_set : 1;
-    if ((st = grow(ctx, (void**)&ctx->d_keys, &ctx->keys_cap, koff * 8 * n_set, true)) != VIO_OK) return st;
-    if ((st = grow(ctx, (void**)&ctx->d_pyr, &ctx->pyr_cap, std::max<size_t>(poff, 256), false)) != VIO_OK) return st;
+    if ((st = grow(ctx, (void**)&ctx->d_keys, &ctx->keys_cap, koff * 8 * n_set, &s)) != VIO_OK) return st;
+    if ((st = grow(ctx, (void**)&ctx->d_pyr, &ctx->pyr_cap, std::max<size_t>(poff, 256))) != VIO_OK) return st;
     if (keys0 != ctx->d_keys || pyr0 != ctx->d_pyr) ctx->map_cache.clear();
 
     VIO_CK(follow_context(ctx, s));
@@ -692,7 +692,7 @@ vio_status plan_staging(vio_ctx* ctx, const uint8_t* const* frames, const vio_di
         }
     }
     vio_status st;
-    if (out->any && (st = grow(ctx, (void**)&ctx->d_in, &ctx->in_cap, need, false)) != VIO_OK) return st;
+    if (out->any && (st = grow(ctx, (void**)&ctx->d_in, &ctx->in_cap, need)) != VIO_OK) return st;
     for (int i = 0; i < n; ++i)
         if (out->src[i]) out->lev0[i] = ctx->d_in + off[i];
     return VIO_OK;
@@ -743,8 +743,8 @@ vio_status detect_in_groups(vio_ctx* ctx, const UploadPlan& plan, const uint8_t*
     // buffer, and a call over the budget ends before any work is enqueued
     const void* keys0 = ctx->d_keys;
     const void* pyr0 = ctx->d_pyr;
-    if ((st = grow(ctx, (void**)&ctx->d_keys, &ctx->keys_cap, keys * 8, true)) != VIO_OK) return st;
-    if ((st = grow(ctx, (void**)&ctx->d_pyr, &ctx->pyr_cap, std::max<size_t>(pyr, 256), false)) != VIO_OK) return st;
+    if ((st = grow(ctx, (void**)&ctx->d_keys, &ctx->keys_cap, keys * 8, &s)) != VIO_OK) return st;
+    if ((st = grow(ctx, (void**)&ctx->d_pyr, &ctx->pyr_cap, std::max<size_t>(pyr, 256))) != VIO_OK) return st;
     if (keys0 != ctx->d_keys || pyr0 != ctx->d_pyr) ctx->map_cache.clear();
     if (!ctx->copy_stream) VIO_CK(cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking));
     for (auto& e : ctx->group_ev)
@@ -824,7 +824,7 @@ vio_status detect_from_host(vio_ctx* ctx, const uint8_t* const* host_frames, con
     // each; so does anything else.
     const UploadPlan plan = plan_upload(host_frames, dims, n);
     vio_status st;
-    if ((st = grow(ctx, (void**)&ctx->d_in, &ctx->in_cap, std::max<size_t>(plan.bytes, 256), false)) != VIO_OK)
+    if ((st = grow(ctx, (void**)&ctx->d_in, &ctx->in_cap, std::max<size_t>(plan.bytes, 256))) != VIO_OK)
         return st;
     std::vector<const uint8_t*> lev0(n), src0(n, nullptr);
     std::vector<int> src_pitch(n, 0);
@@ -980,9 +980,7 @@ vio_status vio_create(vio_ctx** out, const vio_config* cfg_in) {
         cudaEventCreateWithFlags(&ctx->clear_ev, cudaEventDisableTiming) != cudaSuccess)
         return cleanup(VIO_ERR_CUDA);
     if (cudaMalloc(&ctx->d_call, ctx->call_cap) != cudaSuccess) return cleanup(VIO_ERR_OOM);
-    constexpr size_t counter_bytes = 16 + (sizeof(uint64_t) + sizeof(int32_t)) * kTileCap[1];
-    if (cudaMalloc(&ctx->d_counter, counter_bytes) != cudaSuccess) return cleanup(VIO_ERR_OOM);
-    if (clear_buffer(ctx, ctx->d_counter, counter_bytes) != cudaSuccess) return cleanup(VIO_ERR_CUDA);
+    if (cudaMalloc(&ctx->d_counter, kCounterBytes) != cudaSuccess) return cleanup(VIO_ERR_OOM);
     ctx->d_sums = reinterpret_cast<uint64_t*>(ctx->d_counter + 4);
     ctx->d_done = reinterpret_cast<int32_t*>(ctx->d_sums + kTileCap[1]);
     if (cudaHostAlloc(&ctx->h_status, 64, cudaHostAllocMapped) != cudaSuccess) return cleanup(VIO_ERR_OOM);
@@ -1161,7 +1159,7 @@ vio_status vio_detect_host(vio_ctx* ctx, const uint8_t* const* host_frames, cons
         ncell_total += vio_num_cells(dims[i].w, dims[i].h, cell);
     }
     const size_t cell_bytes = ncell_total * sizeof(int4) + align_up(sizeof(int32_t) * n, 16);
-    if ((st = grow(ctx, (void**)&ctx->d_cells, &ctx->cells_cap, cell_bytes, false)) != VIO_OK) return st;
+    if ((st = grow(ctx, (void**)&ctx->d_cells, &ctx->cells_cap, cell_bytes)) != VIO_OK) return st;
     if (ctx->h_out_cap < cell_bytes) {
         if (ctx->h_out) cudaFreeHost(ctx->h_out);
         ctx->h_out = nullptr;
@@ -1224,9 +1222,9 @@ vio_status vio_detect_host_async(vio_ctx* ctx, const uint8_t* const* host_frames
     // the kernels of the slot's previous call have read its frames
     if (slot.used) VIO_CK(cudaStreamWaitEvent(s, slot.done, 0));
     const UploadPlan plan = plan_upload(host_frames, dims, n);
-    if ((st = grow(ctx, (void**)&slot.d_in, &slot.in_cap, std::max<size_t>(plan.bytes, 256), false)) != VIO_OK)
+    if ((st = grow(ctx, (void**)&slot.d_in, &slot.in_cap, std::max<size_t>(plan.bytes, 256))) != VIO_OK)
         return st;
-    if ((st = grow(ctx, (void**)&slot.d_counts, &slot.counts_cap, sizeof(int32_t) * n, false)) != VIO_OK) return st;
+    if ((st = grow(ctx, (void**)&slot.d_counts, &slot.counts_cap, sizeof(int32_t) * n)) != VIO_OK) return st;
     std::vector<const uint8_t*> lev0(n);
     for (int i = 0; i < n; ++i) lev0[i] = slot.d_in + plan.off[i];
     if ((st = enqueue_upload(ctx, plan, slot.d_in, s)) != VIO_OK) return st;

@@ -18,6 +18,9 @@ namespace vio {
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
+constexpr int kTileCap[2] = {8, 64};  // frames of the two forms of tile_detect_kernel
+// d_counter: the work counter (16 bytes), then d_sums and d_done
+constexpr size_t kCounterBytes = 16 + (sizeof(uint64_t) + sizeof(int32_t)) * kTileCap[1];
 constexpr int kMaxCtasPerSm = 4;  // the detect kernels' launch bounds
 
 using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -126,12 +129,14 @@ struct vio_ctx {
     size_t h_out_cap = 0;
 
     cudaEvent_t stage_ev[4] = {nullptr, nullptr, nullptr, nullptr};
-    cudaStream_t capture_stream = nullptr;  // the context's own: graphs are captured and buffers cleared on it
+    cudaStream_t capture_stream = nullptr;  // the context's own: graphs are captured on it
     cudaEvent_t last_ev = nullptr;
     cudaStream_t last_stream = nullptr;
     bool have_last = false;
-    cudaEvent_t clear_ev = nullptr;         // after the latest clear of a buffer (clear_buffer)
-    bool clear_pending = false;             // no call has followed it yet
+    // the latest clear of a buffer, while no call has followed it (clear_buffer)
+    cudaEvent_t clear_ev = nullptr;
+    bool clear_pending = false;
+    bool counters_clear = false;            // d_counter, d_sums and d_done have been cleared
 
     // one graph per (variant, levels, CTAs per SM): every batch shape replays
     // it; CTAs per SM 0 = as many as fit
@@ -196,14 +201,23 @@ inline vio_status fail(vio_ctx* c, vio_status s, const std::string& msg) {
         }                                                                                     \
     } while (0)
 
-// Clears device memory on a stream of the context's own, for kernels enqueued
-// after follow_context: the default stream is not ordered with a caller's
-// non-blocking stream, and what is queued on it is none of the call's business.
-// (Waiting here instead costs a context's first call 10 us.)
-inline cudaError_t clear_buffer(vio_ctx* ctx, void* p, size_t bytes) {
-    cudaError_t e = cudaMemsetAsync(p, 0, bytes, ctx->capture_stream);
-    if (e == cudaSuccess) e = cudaEventRecord(ctx->clear_ev, ctx->capture_stream);
-    if (e == cudaSuccess) ctx->clear_pending = true;
+// Clears device memory for the call on `s`, on that stream: the default stream is
+// not ordered with a caller's non-blocking one.  A later call on another stream
+// waits for the clear (follow_context).  A stream that is being captured would
+// only record it: there it is done at once.
+inline cudaError_t clear_buffer(vio_ctx* ctx, void* p, size_t bytes, cudaStream_t s) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(s, &capture);
+    if (e != cudaSuccess) return e;
+    if (capture != cudaStreamCaptureStatusNone) {
+        e = cudaMemsetAsync(p, 0, bytes, ctx->capture_stream);
+        return e != cudaSuccess ? e : cudaStreamSynchronize(ctx->capture_stream);
+    }
+    if (ctx->clear_pending) e = cudaStreamWaitEvent(s, ctx->clear_ev, 0);
+    if (e == cudaSuccess) e = cudaMemsetAsync(p, 0, bytes, s);
+    if (e == cudaSuccess) e = cudaEventRecord(ctx->clear_ev, s);
+    if (e != cudaSuccess) return e;
+    ctx->clear_pending = true;
     return e;
 }
 
@@ -213,13 +227,12 @@ inline cudaError_t clear_buffer(vio_ctx* ctx, void* p, size_t bytes) {
 inline cudaError_t follow_context(vio_ctx* ctx, cudaStream_t s) {
     cudaError_t e = cudaSuccess;
     if (ctx->have_last && ctx->last_stream != s) e = cudaStreamWaitEvent(s, ctx->last_ev, 0);
-    if (e != cudaSuccess || !ctx->clear_pending) return e;
-    // (a capture cannot wait for work outside it: where one is allowed, the host does)
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    e = cudaStreamIsCapturing(s, &capture);
-    if (e != cudaSuccess) return e;
-    return capture == cudaStreamCaptureStatusNone ? cudaStreamWaitEvent(s, ctx->clear_ev, 0)
-                                                  : cudaEventSynchronize(ctx->clear_ev);
+    if (e == cudaSuccess && ctx->clear_pending) e = cudaStreamWaitEvent(s, ctx->clear_ev, 0);
+    if (e == cudaSuccess && !ctx->counters_clear) {  // the context's first call
+        e = clear_buffer(ctx, ctx->d_counter, kCounterBytes, s);
+        ctx->counters_clear = e == cudaSuccess;
+    }
+    return e;
 }
 
 inline cudaError_t mark_last(vio_ctx* ctx, cudaStream_t s) {
@@ -233,7 +246,9 @@ inline cudaError_t mark_last(vio_ctx* ctx, cudaStream_t s) {
 
 // Grows a resident buffer to `need` bytes.  Growing waits for the device
 // (the old buffer may still be in use), so buffers grow geometrically.
-inline vio_status grow(vio_ctx* ctx, void** p, size_t* cap, size_t need, bool zero) {
+// With clear_for the new buffer is zero for calls that follow_context, the first
+// of them on that stream.
+inline vio_status grow(vio_ctx* ctx, void** p, size_t* cap, size_t need, const cudaStream_t* clear_for = nullptr) {
     if (need <= *cap && *p) return VIO_OK;
     size_t want = std::max(need, *cap + *cap / 2);
     const size_t budget = ctx->cfg.mem_budget_bytes;
@@ -250,7 +265,7 @@ inline vio_status grow(vio_ctx* ctx, void** p, size_t* cap, size_t need, bool ze
         *cap = 0;
     }
     VIO_CK(cudaMalloc(p, want));
-    if (zero) VIO_CK(clear_buffer(ctx, *p, want));
+    if (clear_for) VIO_CK(clear_buffer(ctx, *p, want, *clear_for));
     *cap = want;
     ctx->bytes_in_use += want;
     return VIO_OK;

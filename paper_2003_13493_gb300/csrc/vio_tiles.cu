@@ -113,8 +113,8 @@ vio_status detect_form(vio_ctx* ctx, const uint8_t* const* lev0, const int* pitc
     vio_status st;
     const void* keys0 = ctx->d_keys;
     const void* pyr0 = ctx->d_pyr;
-    if ((st = grow(ctx, (void**)&ctx->d_keys, &ctx->keys_cap, koff * 8, true)) != VIO_OK) return st;
-    if ((st = grow(ctx, (void**)&ctx->d_pyr, &ctx->pyr_cap, std::max<size_t>(poff, 256), false)) != VIO_OK) return st;
+    if ((st = grow(ctx, (void**)&ctx->d_keys, &ctx->keys_cap, koff * 8, &s)) != VIO_OK) return st;
+    if ((st = grow(ctx, (void**)&ctx->d_pyr, &ctx->pyr_cap, std::max<size_t>(poff, 256))) != VIO_OK) return st;
     if (keys0 != ctx->d_keys || pyr0 != ctx->d_pyr) ctx->map_cache.clear();
     koff = 0;
     poff = ctx->group_pyr0;

@@ -25,7 +25,6 @@ struct TileCall {
     int32_t tiles[kMaxLevels * CAP + 1];  // prefix sums: entry j * n + f is level top - j of frame f
     FrameDesc f[CAP];
 };
-constexpr int kTileCap[2] = {8, 64};  // frames of the two forms
 static_assert(sizeof(TileCall<64>) <= 16384, "kernel parameter");
 
 // A level in memory.

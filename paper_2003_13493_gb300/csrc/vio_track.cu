@@ -198,8 +198,8 @@ vio_status track_impl(vio_ctx* ctx, const uint8_t* const* prev, const uint8_t* c
     if (!T.done_ev) VIO_CK(cudaEventCreateWithFlags(&T.done_ev, cudaEventDisableTiming));
     // the previous call's kernels read the device buffers this call rewrites
     if (T.have_done) VIO_CK(cudaStreamWaitEvent(s, T.done_ev, 0));
-    if ((st = grow(ctx, (void**)&T.d_in, &T.in_cap, std::max<size_t>(ioff, 256), false)) != VIO_OK) return st;
-    if ((st = grow(ctx, (void**)&T.d_pyr, &T.pyr_cap, std::max<size_t>(poff, 256), false)) != VIO_OK) return st;
+    if ((st = grow(ctx, (void**)&T.d_in, &T.in_cap, std::max<size_t>(ioff, 256))) != VIO_OK) return st;
+    if ((st = grow(ctx, (void**)&T.d_pyr, &T.pyr_cap, std::max<size_t>(poff, 256))) != VIO_OK) return st;
     if (n_pairs <= 8) {
         if ((st = track_launch<8>(ctx, p, frames.data(), dims, 0, n_pairs, pts, n_pts, out, cells_in, s)) != VIO_OK)
             return st;

@@ -25,6 +25,7 @@ std::map<uintptr_t, size_t> g_pinned;              // page-locked ranges
 std::map<std::string, int> g_fail;                 // op -> calls until it fails
 cudaStream_t g_capturing = nullptr;
 bool g_any_capture = false;
+cudaStream_t g_begun = nullptr;                    // stream whose work the library itself captures
 uintptr_t g_next = 1;
 struct { dim3 grid, block; size_t smem; cudaStream_t stream; } g_config;
 
@@ -58,7 +59,7 @@ void* room(size_t n) {
 
 cudaError_t launch(const void* f, cudaStream_t s) {
     if (fails("launch")) return cudaErrorLaunchFailure;
-    note("launch %p %s", (void*)s, kernels().count(f) ? kernels()[f].c_str() : "?");
+    note(s == g_begun && s ? "captured %p %s" : "launch %p %s", (void*)s, kernels().count(f) ? kernels()[f].c_str() : "?");
     return cudaSuccess;
 }
 
@@ -227,8 +228,12 @@ cudaError_t cudaStreamIsCapturing(cudaStream_t s, cudaStreamCaptureStatus* st) {
     *st = capturing(s) ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
     return cudaSuccess;
 }
-cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { return cudaSuccess; }
+cudaError_t cudaStreamBeginCapture(cudaStream_t s, cudaStreamCaptureMode) {
+    g_begun = s;
+    return cudaSuccess;
+}
 cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t* g) {
+    g_begun = nullptr;
     *g = (cudaGraph_t)g_next++;
     return cudaSuccess;
 }

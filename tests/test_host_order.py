@@ -169,7 +169,7 @@ def test_cleared_buffers_are_ready_on_any_stream(host, sizes):
         for s, first in launches.items():
             if c < first:
                 assert ordered(log, c, first), (log[c], hex(s))
-    assert clears[0] < clears[1] < launches[S1] < clears[2] < launches[S2]
+    assert max(clears[:2]) < launches[S1] < clears[2] < launches[S2]
 
 
 @pytest.mark.parametrize("small", [[(640, 480)], [(160, 120)] * 70], ids=["tiles", "persistent"])
