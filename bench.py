@@ -397,7 +397,7 @@ def run_ours(args, rank, world, local_rank):
     if sweep:
         res["detections_per_s"] = round(world * n * npar * args.steps / (ms / 1e3), 1)
     if not args.no_extras and not sweep:
-        res["e2e"] = e2e_leg(args, wl, det, dev, stream, frames_np, dims, n, world)
+        res["e2e"] = e2e_leg(args, wl, dev, stream, frames_np, dims, n, world)
     if world > 1:
         args.no_cpu_baseline = True  # the oracle baseline is an N = 1 figure
     if rank == 0 and not args.no_extras:
@@ -419,7 +419,7 @@ def run_ours(args, rank, world, local_rank):
     return res
 
 
-def e2e_leg(args, wl, det, dev, stream, frames_np, dims, n, world) -> dict:
+def e2e_leg(args, wl, dev, stream, frames_np, dims, n, world) -> dict:
     """End to end through the host-buffer entry points (pinned host frames and
     outputs): each step copies its frames in and its records out.  Every rank
     runs it on its own GPU; the whole-job rate divides all ranks' frames by
@@ -444,8 +444,11 @@ def e2e_leg(args, wl, det, dev, stream, frames_np, dims, n, world) -> dict:
              for w, h in dims]
         return o, torch.empty(n, dtype=torch.int32).pin_memory().numpy()
 
+    # as a user's context: a pinned variant would keep its calls with the
+    # persistent kernels, in one piece
     e2e_det = vio.Detector(device=dev.index, max_frames=max(64, n))
-    e2e_det.set_variant(det.tuning()[2])
+    if args.variant >= 0:
+        e2e_det.set_variant(args.variant)
     esteps = max(3, min(args.steps, 50))
     streams = [torch.cuda.Stream(device=dev), torch.cuda.Stream(device=dev)]
     bufs = [pinned_outs(), pinned_outs()]
@@ -644,7 +647,8 @@ def extras(args, wl, det, dev, stream, sh, frames_np, dims, marshalled, optr, cp
 
     # plain path: one frame per call
     plain = vio.Detector(device=dev.index, max_frames=4)
-    plain.set_variant(det.tuning()[2])
+    if args.variant >= 0:  # (a pinned variant keeps a call with the persistent kernels)
+        plain.set_variant(args.variant)
     single = [((ctypes.c_void_p * 1)(marshalled[s][0][i]), (vio.Dims * 1)(marshalled[s][1][i]),
                (ctypes.c_void_p * 1)(optr[i])) for s in range(len(marshalled)) for i in range(n)]
     psteps = max(3, min(args.steps, 100))
@@ -663,7 +667,7 @@ def extras(args, wl, det, dev, stream, sh, frames_np, dims, marshalled, optr, cp
     pms = e0.elapsed_time(e1)
     plain.close()
     out["plain"] = {"value": round(psteps * n / (pms / 1e3), 1), "unit": "frames/s",
-                    "what": "same frames, one vio_detect call (and graph replay) per frame"}
+                    "what": "same frames, one vio_detect call per frame"}
 
     out["latency"] = latency_leg(args, dev.index)
     if args.serve_seconds > 0:
