@@ -117,9 +117,10 @@ __device__ __forceinline__ int upper_index(const int32_t* a, int n, int v) {
 // one level (L = 1) that is all it does.
 //
 // Bound by memory latency and issue on batches of a few tens of megabytes, by
-// HBM on large ones (32 4K frames: 353 MB in 63 us, 0.83 of the copy rate).
-// 24 frames of odd width, 18 MB, 4 levels: 180.6 -> 84.8 us a call with the
-// copies gone; 64 mixed frames 145.5 -> 140.6 us.
+// HBM on large ones (32 4K frames: 353 MB in 63 us, 0.83 of the copy rate).  64
+// mixed frames, 3 levels: 17.6 us alone (20.2 with blocks of 512 columns), 22 us in
+// the call.  24 frames of odd width, 4 levels, by the persistent kernels: 83.6 us a
+// call (180.6 with a copy per frame).
 // ---------------------------------------------------------------------------
 __host__ __device__ constexpr int pyr_rows(int levels) { return levels == 1 ? 4 : 1 << (levels - 1); }
 
@@ -513,10 +514,10 @@ __device__ __forceinline__ uint32_t run_of_even(const uint32_t (&f)[8]) {
 // of every row, and each of the 8 consumer warps owns a band of consecutive
 // rows.
 // Per item:
-//   1. The producer (one thread) claims the item, computes its constants
-//      and TMA loads the region plus the 3-pixel circle halo (box 144 x
-//      TH+2R+6) into one of two image buffers; the other buffer is loading
-//      the next item meanwhile.
+//   1. The producer (one warp) claims the item, decodes it, computes its
+//      constants and TMA loads the region plus the 3-pixel circle halo (box
+//      144 x TH+2R+6) into one of two image buffers; the other buffer is
+//      loading the next item meanwhile (produce_tiles).
 //   2. Coarse test on every score-region pixel of the warp's band, 4 pixels
 //      per lane (runs of the eight even circle points), pixels outside the
 //      testable area masked off; one warp
@@ -647,7 +648,7 @@ __device__ __forceinline__ uint32_t nibble(uint32_t keep) { return (keep * 0x002
 // (logic, shifts, permutes: one instruction every two cycles) and by issue,
 // and this test is half of its ALU work: with the rule and the shuffles per
 // row the mixed batch took 107.1 M warp instructions and 133.7 us, so 94.0 M
-// and 117.5 us; 9x9 NMS at n = 10 on 16 frames 67.6 -> 52.8 us a call.
+// and 117.5 us (96.7 M and 120 us with the producer's whole-warp decoding).
 // Lane 0 has no lane to its left: its W flags of columns 0..2 and NW / SW
 // flags of columns 0, 1 count as set, which keeps more, never fewer.
 //
@@ -831,8 +832,8 @@ __device__ __forceinline__ bool own_rows_reset(uint64_t* nms_bars, int t, T* til
 // 2,400 cycles by one thread and after the release, which the consumers then
 // waited for on top of the load itself: 2,100 of 7,950 cycles per tile on 4K
 // frames with few corners.  It is done by the warp and before the wait for the
-// release (8 4K frames, FAST-12: 107.5 -> 101.8 us a call; 64 mixed frames
-// 148.3 -> 145.5 us).
+// release (8 4K frames, FAST-12: 107.5 -> 101.8 us a call, 96 now; 64 mixed
+// frames 148.3 -> 145.5 us, 138 now).
 //
 // The pyramid's levels are written by the kernel before this one, which may
 // still be running (programmatic dependent launch); a level-0 tile reads the

@@ -52,27 +52,33 @@ void (*pyramid_of(int levels))(TileCall<CAP>) {
 }
 
 // Which calls are taken, by their tiles (of the form in question); us per call,
-// the persistent three kernels against these launches:
-//   form 0, one launch     752x480, 3 levels, 280 tiles of 30 rows: 22.7 -> 10.6
-//                          1280x720: 20.4 -> 12.3; form 1 there 14.4 and 15.4
-//                          (but 8 frames 752x480, 1,200 tiles: form 1 17.0, form 0 20.6)
+// three sets of frames in turn, the persistent three kernels -> these launches:
+//   form 0, one launch, tiles of 30 rows at 3 levels
+//                          752x480, 152 tiles: 20.3 -> 12.3; 1280x720, 354: 22.5 -> 12.3; 1920x1080,
+//                          756: 26.1 -> 15.6; form 1 there 14.9, 16.4 and 18.5.  (The line is the last-tile
+//                          decode's below; with a decode launch form 0 would still be ahead above it:
+//                          8 frames 752x480, 1,216 tiles: 16.9, form 1 18.5.)
 //   form 1, tiles of level 1 and 2 built from level 0
-//                          16 mixed frames, 3 levels, 2,788 tiles: 60.4 -> 39.3; 32, 5,576 tiles:
-//                          84.5 -> 72.5; 48, 8,364 tiles: 111.0 -> 109.1; 64, 11,152 tiles: 138.7 -> 143
+//                          16 mixed frames, 3 levels, 2,788 tiles: 56.7 -> 41.0; 32, 5,576 tiles:
+//                          84.4 -> 77.7; 48, 8,364 tiles: 115.6 -> 113.3; 64, 11,152 tiles: 145.7 -> 150.0
 //   form 1, levels in two launches (more than 3 levels, or unaligned frames)
-//                          4 4K frames, 4 levels, 6,000 tiles: 63.6 -> 61.3; 6, 8,880 tiles: 72.8 -> 76.8;
-//                          6 of 3001x2001, 6,694 tiles: 115.1 -> 103.9; 48 of 1021x765, 7,595: 125.0 -> 122.6;
-//                          (16 and 48 mixed frames, 3 levels: 46.0 and 110.0)
+//                          aligned: 4 4K frames, 4 levels, 6,000 tiles: 57.9 -> 57.2; 5, 7,500 tiles:
+//                          69.7 -> 68.2; 6, 9,000 tiles: 79.4 -> 79.9
+//                          unaligned: 24 of 1021x765 and less, 4 levels, 3,902 tiles: 83.6 -> 72.6; 48,
+//                          7,777 tiles: 140.9 -> 128.0; 6 of 3001x2001, 3 levels, 6,852 tiles: 94.3 -> 89.4
+//                          (8, 9,136 tiles, would be 117.7 -> 113.7)
+//                          (aligned, 3 levels: 16, 32 and 48 mixed frames 47.2, 80.7 and 112.9)
 //   form 1 after a pyramid kernel that uploads the frames
-//                          16 pinned frames, host call: 140 -> 127; 8: 87.5 -> 82
-// (a tile costs more here, 11 to 13 us per 1,000 of the mixed frames' against 9.4 in
-// the persistent kernel, whose loads run ahead; a call costs up to 27 us less to start).
+//                          host call, pinned frames apart, 3 levels: 8 mixed 90.2 -> 82.8; 16: 142.7 ->
+//                          130.8; 32: 242.6 -> 235.6
+// (a tile costs more here, 13.0 us per 1,000 of the mixed frames' against 10.6 in the
+// pyramid and persistent kernels, whose loads run ahead; a call costs 8 to 22 us less to start).
 constexpr int kFormTiles[2] = {800, 8000};      // aligned frames, at most 3 levels
 constexpr int kTwoStepTiles[2] = {6000, 8000};  // others: aligned, unaligned
 // A frame is decoded by the CTA of its last tile in a call of at most this many
 // tiles; above it a decode launch is faster than a fence and a count per tile
-// (8 1920x1080 frames, 3,040 tiles: 45.3 -> 42.5 us; 64 of 320x240, 1,088 tiles:
-// 22.7 either way).
+// (8 1920x1080 frames, 3,040 tiles of 62 rows: 46.2 -> 43.2 us; 64 of 320x240, 1,088
+// tiles: 22.6 and 22.5; one 752x480 frame in form 0: 12.3 either way).
 constexpr int kLastTileDecodes = 800;
 
 int tiles_of(const vio_dims& d, int k, int th) {

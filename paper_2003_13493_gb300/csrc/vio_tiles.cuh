@@ -118,11 +118,11 @@ __device__ __forceinline__ void emit_levels(const FrameDesc& fd, const ItemInfo&
     }
 }
 
-// One CTA of 8 warps per tile, five CTAs per SM (48 registers, 43 KB; three and
-// four per SM: 51.2 and 46.4 us instead of 43.1 for 16 mixed frames).
+// One CTA of 8 warps per tile, five CTAs per SM (48 registers, 43 KB; with four,
+// 43.0 us a call instead of 41.0 for 16 mixed frames, 79.8 instead of 77.5 for 32).
 //
 // The persistent kernel between a pyramid and a decode kernel costs a call about
-// 34 us whatever its size: the call block's upload, three launches, the ramp
+// 20 us whatever its size: the call block's upload, three launches, the ramp
 // and the tail of each.  Here
 //  - with up to 3 levels all tiles are one launch: a tile of level 1 or 2
 //    builds its box from level 0 (with its halo, 1.35 times the level-0 bytes
@@ -137,9 +137,9 @@ __device__ __forceinline__ void emit_levels(const FrameDesc& fd, const ItemInfo&
 // its CTAs move in as that drains.
 // The phases of a tile are separated by CTA barriers, and the other four CTAs of
 // the SM fill them.  A tile alone takes 3.4 us (load 1.3, coarse test 0.6, full
-// test, scores and NMS 0.6, fence and count 0.9); the 280 tiles of a 752x480
-// frame, 8 us with the decode.  The rule for which calls come here stands in
-// vio_tiles.cu.
+// test, scores and NMS 0.6, fence and count 0.9); one 752x480 frame, 152 tiles of
+// 30 rows, 10.3 us a call with the decode.  The rule for which calls come here
+// stands in vio_tiles.cu.
 template <int TH, int MODE, int R, int CAP>
 __global__ void __launch_bounds__(kConsumers, 5) tile_detect_kernel(const __grid_constant__ TileCall<CAP> call) {
     using G = TileGeom<TH, R>;
